@@ -155,8 +155,8 @@ typedef struct {
 typedef struct asap_moe_s* asap_moe_t;
 
 /* Validate cfg, allocate the handle's device memory on the current device,
- * copy and pack the weights (gate/up rows interleaved in blocks of 128 so one
- * 256-wide GEMM tile holds matching gate and up columns) and build the weight
+ * copy and pack the weights (gate/up rows interleaved so one 256-wide GEMM
+ * tile holds matching gate and up columns) and build the weight
  * TMA descriptors.  Synchronous: it first synchronises the device, so weights
  * still being written on any stream are complete before they are read.  On
  * failure *out is NULL. */
@@ -185,13 +185,15 @@ int asap_moe_n_layers(asap_moe_t h, int32_t* n_layers);
 
 /* Tile shape of the BF16 grouped expert GEMMs (gate/up and down) of the
  * calls that follow on this handle (the FP8 GEMMs have one shape):
- *  - ASAP_TILING_AUTO (the default): per launch, paired tiles when the
- *    routed rows average at least 128 per expert and the launch has at least
- *    three waves of paired tiles (estimated from n, top_k and the expert
- *    count; one tile per SM per wave), else single tiles.
- *  - ASAP_TILING_SINGLE: 128-row m-tiles.
- *  - ASAP_TILING_PAIRED: two 128-row m-tiles of one expert per tile, sharing
- *    every weight box; a segment's last <= 128 rows form a half tile.
+ *  - ASAP_TILING_AUTO (the default): per launch, CTA pairs when the routed
+ *    rows average at least 64 per expert or the launch has at most two waves
+ *    of single-CTA tiles (from n, top_k and the expert count), else single
+ *    CTAs.
+ *  - ASAP_TILING_SINGLE: one CTA per tile, tiles of 128 rows.
+ *  - ASAP_TILING_PAIRED: two CTAs on the SMs of one TPC per tile, tiles of up
+ *    to 256 rows of one expert (equal heights within a segment, in steps of
+ *    32).  (The fused combine below runs single CTAs in every mode, with two
+ *    128-row m-tiles per tile under this one.)
  * Every mode computes each output element with the same products in the same
  * order, so the results are bit-identical; only the speed differs.  Another
  * mode returns ASAP_ERR_INVALID.  Host state only (nothing is enqueued); do

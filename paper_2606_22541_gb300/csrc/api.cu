@@ -317,8 +317,9 @@ int run_route(asap_moe_t h, const void* x, int n, int32_t* idx, float* w, int32_
   return run_gate_scan(h, logits, splits, n, idx, w, counts, offsets, ws, layer, st);
 }
 
-// Paired m-tiles (two 128-row m-tiles per GEMM tile sharing the weight
-// boxes, a half tile for a segment's last <= 128 rows) when
+// Paired m-tiles of the down GEMM with the fused combine (two 128-row m-tiles
+// per GEMM tile sharing the weight boxes, a half tile for a segment's last
+// <= 128 rows) when
 //  - the segments hold at least one m-tile (128 rows) per expert on average:
 //    below that nearly every paired tile is a half tile, and the paired rings
 //    (3 + 3 stages) keep fewer weight bytes in flight than the single-tile
@@ -348,6 +349,76 @@ int ub_mtiles(const asap_moe_config& c, long long nk, int bm = asap::kGemmBM) {
 // warp's 32 rows).
 constexpr uint32_t kStoreRows = 32;
 
+// Launch of a bf16 expert GEMM: A operands in0 [nk, K0] and in1 [n, K1] (the
+// shared expert's, when a.m1 > 0), outputs a.out0 and a.out1.
+int launch_expert_gemm(asap_moe_t h, int epi, bool cta2, bool pair, const void* in0, long long nk, int K0,
+                       const void* in1, int n, int K1, asap::GemmArgs& a, cudaStream_t st) {
+  const bool sh = a.m1 > 0;
+  std::string err;
+  bool ok = true;
+  auto enc = [&](CUtensorMap* m, const void* p, long long rows, long long cols, uint32_t box) {
+    ok = ok && asap::encode_tmap_bf16(m, p, rows, cols, box, &err);
+  };
+  if (cta2) {
+    CUtensorMap maps[10];
+    for (int i = 0; i < 4; ++i) {
+      enc(&maps[i], in0, nk, K0, 32 * (i + 1));
+      if (sh) enc(&maps[4 + i], in1, n, K1, 32 * (i + 1));
+      else maps[4 + i] = maps[i];
+    }
+    enc(&maps[8], a.out0, nk, a.ldo0, kStoreRows);
+    if (sh) enc(&maps[9], a.out1, n, a.ldo1, kStoreRows);
+    else maps[9] = maps[8];
+    if (!ok) return fail(ASAP_ERR_INVALID, "expert GEMM operand: " + err);
+    a.bmap0 += asap::MAP_PAIR;
+    a.bmap1 += asap::MAP_PAIR;
+    const long long tiles = static_cast<long long>(ub_mtiles(h->cfg, nk, 256)) * a.n_tiles0 +
+                            (sh ? static_cast<long long>(asap::ceil_div(n, 256)) * a.n_tiles1 : 0);
+    CU_TRY(asap::pair_gemm_launch(epi, maps, a, static_cast<int>(std::min<long long>(tiles, h->num_sms / 2)), st),
+           "expert GEMM launch");
+    return ASAP_OK;
+  }
+  CUtensorMap maps[4];
+  enc(&maps[0], in0, nk, K0, asap::kGemmBM);
+  enc(&maps[2], a.out0, nk, a.ldo0, kStoreRows);
+  if (sh) {
+    enc(&maps[1], in1, n, K1, asap::kGemmBM);
+    enc(&maps[3], a.out1, n, a.ldo1, kStoreRows);
+  } else {
+    maps[1] = maps[0];
+    maps[3] = maps[2];
+  }
+  if (!ok) return fail(ASAP_ERR_INVALID, "expert GEMM operand: " + err);
+  const int bm = pair ? 2 * asap::kGemmBM : asap::kGemmBM;
+  const long long tiles = static_cast<long long>(ub_mtiles(h->cfg, nk, bm)) * a.n_tiles0 +
+                          (sh ? static_cast<long long>(asap::ceil_div(n, bm)) * a.n_tiles1 : 0);
+  CU_TRY(asap::gemm_launch(epi, pair, maps, a, static_cast<int>(std::min<long long>(tiles, h->num_sms)), st),
+         "expert GEMM launch");
+  return ASAP_OK;
+}
+
+// CTA pairs (gemm_pair.cu) when the segments hold at least 64 rows per expert
+// on average, or when the launch has at most two waves of single-CTA tiles.
+// Measured on a GB300 (gate/up | down us, pairs vs single CTAs):
+//  - DeepSeek-V3, balanced: 8192 tokens 3059 | 1692 vs 3590 | 1915, 4096
+//    tokens (128 rows per expert) 2327 | 1238 vs 2416 | 1282; below the line
+//    both stream the weights at the HBM rate and the single CTAs' larger boxes
+//    are a little ahead: 1024 tokens (32 rows) 2110 | 1102 vs 2099 | 1082;
+//  - Mixtral 1536 tokens 455 | 258 vs 551 | 275, 128 tokens (32 rows)
+//    268 | 144 vs 265 | 141;
+//  - DeepSeek-V3, 1 token (9 experts, 144 gate/up tiles): 86 | 53 vs 109 | 65,
+//    two half-length waves of pairs instead of one wave of single CTAs.
+// Short contractions stay on single CTAs: a pair's set-up costs about 1 us more
+// (the tiny layer, K = 256 and 128: 41.6 vs 39.7 us for the whole layer).
+bool use_cta2(asap_moe_t h, long long nk, int n_tiles0, long long m1, int n_tiles1, int k_iters) {
+  if (h->tiling != ASAP_TILING_AUTO) return h->tiling == ASAP_TILING_PAIRED;
+  if (k_iters < 16) return false;
+  if (nk >= 64ll * h->cfg.n_experts) return true;
+  const long long tiles = std::min<long long>(h->cfg.n_experts, nk) * n_tiles0 +
+                          static_cast<long long>(asap::ceil_div(m1, asap::kGemmBM)) * n_tiles1;
+  return tiles <= 2ll * h->num_sms;
+}
+
 // GEMM1: h = silu(X Wg^T) * (X Wu^T) on the routed segments, plus the shared
 // expert on x (problem 1 of the same launch).
 // counter: a zeroed int the launch claims its tiles from (nullptr: static order).
@@ -359,23 +430,6 @@ int run_gate_up(asap_moe_t h, const void* x_perm, const int32_t* offsets, const 
   const asap_moe_config& c = h->cfg;
   const long long nk = static_cast<long long>(n) * c.top_k;
   const bool sh = c.n_shared != 0;
-  const bool pair = use_pair(h, nk, c.inter / 128, sh ? n : 0, c.shared_inter / 128);
-  const int bm = pair ? 2 * asap::kGemmBM : asap::kGemmBM;
-  std::string err;
-  CUtensorMap maps[4];
-  if (!asap::encode_tmap_bf16(&maps[0], x_perm, nk, c.hidden, asap::kGemmBM, &err))
-    return fail(ASAP_ERR_INVALID, "x_perm: " + err);
-  if (!asap::encode_tmap_bf16(&maps[2], hbuf, nk, c.inter, kStoreRows, &err))
-    return fail(ASAP_ERR_INVALID, "h: " + err);
-  if (sh) {
-    if (!asap::encode_tmap_bf16(&maps[1], x, n, c.hidden, asap::kGemmBM, &err))
-      return fail(ASAP_ERR_INVALID, "x: " + err);
-    if (!asap::encode_tmap_bf16(&maps[3], hsh, n, c.shared_inter, kStoreRows, &err))
-      return fail(ASAP_ERR_INVALID, "h_shared: " + err);
-  } else {
-    maps[1] = maps[0];
-    maps[3] = maps[2];
-  }
   asap::GemmArgs a{};
   a.lref = lref(h, layer);
   a.bmap0 = asap::MAP_GATE_UP;
@@ -400,12 +454,8 @@ int run_gate_up(asap_moe_t h, const void* x_perm, const int32_t* offsets, const 
   a.k_splits = 1;
   a.tile_counter = counter;
   a.b_tiled = 1;  // weights in tile-contiguous order (pack_layer)
-  const long long tiles = static_cast<long long>(ub_mtiles(c, nk, bm)) * a.n_tiles0 +
-                          (sh ? static_cast<long long>(asap::ceil_div(n, bm)) * a.n_tiles1 : 0);
-  CU_TRY(asap::gemm_launch(asap::EPI_SWIGLU, pair, maps, a, static_cast<int>(std::min<long long>(tiles, h->num_sms)),
-                           st),
-         "gate/up GEMM launch");
-  return ASAP_OK;
+  const bool cta2 = use_cta2(h, nk, a.n_tiles0, a.m1, a.n_tiles1, a.k_iters0);
+  return launch_expert_gemm(h, asap::EPI_SWIGLU, cta2, false, x_perm, nk, c.hidden, x, n, c.hidden, a, st);
 }
 
 // GEMM2: y = h Wd^T on the routed segments, plus the shared expert.
@@ -426,23 +476,6 @@ int run_down(asap_moe_t h, const void* hbuf, const int32_t* offsets, const void*
   const asap_moe_config& c = h->cfg;
   const long long nk = static_cast<long long>(n) * c.top_k;
   const bool sh = c.n_shared != 0;
-  const bool pair = use_pair(h, nk, c.hidden / asap::kGemmBN, sh ? n : 0, c.hidden / asap::kGemmBN);
-  const int bm = pair ? 2 * asap::kGemmBM : asap::kGemmBM;
-  std::string err;
-  CUtensorMap maps[4];
-  if (!asap::encode_tmap_bf16(&maps[0], hbuf, nk, c.inter, asap::kGemmBM, &err))
-    return fail(ASAP_ERR_INVALID, "h: " + err);
-  if (!asap::encode_tmap_bf16(&maps[2], y_perm, nk, c.hidden, kStoreRows, &err))
-    return fail(ASAP_ERR_INVALID, "y_perm: " + err);
-  if (sh) {
-    if (!asap::encode_tmap_bf16(&maps[1], hsh, n, c.shared_inter, asap::kGemmBM, &err))
-      return fail(ASAP_ERR_INVALID, "h_shared: " + err);
-    if (!asap::encode_tmap_bf16(&maps[3], y_sh, n, c.hidden, kStoreRows, &err))
-      return fail(ASAP_ERR_INVALID, "y_shared: " + err);
-  } else {
-    maps[1] = maps[0];
-    maps[3] = maps[2];
-  }
   asap::GemmArgs a{};
   a.lref = lref(h, layer);
   a.bmap0 = asap::MAP_DOWN;
@@ -474,11 +507,10 @@ int run_down(asap_moe_t h, const void* hbuf, const int32_t* offsets, const void*
   a.comb_out = cf.out;
   a.comb_n = n;
   a.comb_k = c.top_k;
-  const long long tiles = static_cast<long long>(ub_mtiles(c, nk, bm)) * a.n_tiles0 +
-                          (sh ? static_cast<long long>(asap::ceil_div(n, bm)) * a.n_tiles1 : 0);
-  CU_TRY(asap::gemm_launch(asap::EPI_BF16, pair, maps, a, static_cast<int>(std::min<long long>(tiles, h->num_sms)), st),
-         "down GEMM launch");
-  return ASAP_OK;
+  // the fused combine runs in the single-CTA kernel's epilogue
+  const bool pair = use_pair(h, nk, a.n_tiles0, a.m1, a.n_tiles1);
+  const bool cta2 = !cf.cnt && use_cta2(h, nk, a.n_tiles0, a.m1, a.n_tiles1, a.k_iters0);
+  return launch_expert_gemm(h, asap::EPI_BF16, cta2, cf.cnt && pair, hbuf, nk, c.inter, hsh, n, c.shared_inter, a, st);
 }
 
 // counters: kTileCounters zeroed ints (or nullptr)
@@ -706,24 +738,26 @@ int pack_layer(asap_moe_t h, const asap_moe_weights* wts, LayerWeights& L, cudaS
     if ((e = cudaMemcpyAsync(L.router_bias, wts->router_bias, E * 4, cudaMemcpyDeviceToDevice, st)) != cudaSuccess)
       return cuda_fail(e, "copy bias");
   }
-  // expert weights in the tile-contiguous order of the GEMMs' weight boxes
-  // (gate/up interleaved per 128 rows), so each box is one 32 KB read
+  // expert weights in the tile-contiguous order of the GEMMs' weight boxes, so
+  // each box is one 32 KB read; gate/up rows alternate in eights (bf16) or per
+  // 128 rows (FP8)
+  const int log_unit = h->fp8 ? 7 : 3;  // log2 of the rows
   if ((e = cudaMalloc(&L.gate_up, gu_bytes)) != cudaSuccess) return cuda_fail(e, "cudaMalloc gate/up");
   if ((e = asap::launch_retile(wts->w_gate, wts->w_up, static_cast<int>(E), static_cast<int>(2 * I),
-                               static_cast<long long>(H * wb), true, L.gate_up, st)) != cudaSuccess)
+                               static_cast<long long>(H * wb), true, log_unit, L.gate_up, st)) != cudaSuccess)
     return cuda_fail(e, "pack gate/up");
   if ((e = cudaMalloc(&L.down, down_bytes)) != cudaSuccess) return cuda_fail(e, "cudaMalloc down");
   if ((e = asap::launch_retile(wts->w_down, nullptr, static_cast<int>(E), static_cast<int>(H),
-                               static_cast<long long>(I * wb), false, L.down, st)) != cudaSuccess)
+                               static_cast<long long>(I * wb), false, log_unit, L.down, st)) != cudaSuccess)
     return cuda_fail(e, "pack down");
   if (c.n_shared) {
     if ((e = cudaMalloc(&L.sh_gate_up, 2 * Is * H * wb)) != cudaSuccess) return cuda_fail(e, "cudaMalloc shared");
     if ((e = asap::launch_retile(wts->sh_gate, wts->sh_up, 1, static_cast<int>(2 * Is), static_cast<long long>(H * wb),
-                                 true, L.sh_gate_up, st)) != cudaSuccess)
+                                 true, log_unit, L.sh_gate_up, st)) != cudaSuccess)
       return cuda_fail(e, "pack shared");
     if ((e = cudaMalloc(&L.sh_down, H * Is * wb)) != cudaSuccess) return cuda_fail(e, "cudaMalloc shared down");
     if ((e = asap::launch_retile(wts->sh_down, nullptr, 1, static_cast<int>(H), static_cast<long long>(Is * wb), false,
-                                 L.sh_down, st)) != cudaSuccess)
+                                 log_unit, L.sh_down, st)) != cudaSuccess)
       return cuda_fail(e, "pack shared down");
   }
   if (h->fp8) {
@@ -769,8 +803,12 @@ int encode_layer(asap_moe_t h, const LayerWeights& L, asap::LayerEntry* out) {
   const uint64_t wb = h->fp8 ? 1 : 2;
   auto enc = [&](int which, const void* p, uint64_t rows, uint64_t cols) {
     const uint64_t rows128 = rows * cols * wb / 128;
-    return h->fp8 ? asap::encode_tmap_u8(&out->map[which], p, rows128, 128, asap::kGemmBN, &err)
-                  : asap::encode_tmap_bf16(&out->map[which], p, rows128, 64, asap::kGemmBN, &err);
+    CUtensorMap* m = &out->map[which];
+    CUtensorMap* mp = &out->map[asap::MAP_PAIR + which];
+    return h->fp8 ? asap::encode_tmap_u8(m, p, rows128, 128, asap::kGemmBN, &err) &&
+                        asap::encode_tmap_u8(mp, p, rows128, 128, asap::kGemmBN / 2, &err)
+                  : asap::encode_tmap_bf16(m, p, rows128, 64, asap::kGemmBN, &err) &&
+                        asap::encode_tmap_bf16(mp, p, rows128, 64, asap::kGemmBN / 2, &err);
   };
   if (!enc(asap::MAP_GATE_UP, L.gate_up, E * 2 * I, H)) return fail(ASAP_ERR_CUDA, "gate/up map: " + err);
   if (!enc(asap::MAP_DOWN, L.down, E * H, I)) return fail(ASAP_ERR_CUDA, "down map: " + err);
@@ -825,6 +863,7 @@ ASAP_API int asap_moe_create_layers(const asap_moe_config* cfg, const asap_moe_w
     return bail(fail(ASAP_ERR_UNSUPPORTED, "libasap_moe is built for sm_103a (GB300) only; device is sm_" +
                                                std::to_string(cc_major) + std::to_string(cc_minor)));
   e = asap::gemm_set_attributes();
+  if (e == cudaSuccess) e = asap::pair_gemm_set_attributes();
   if (e == cudaSuccess) e = asap::fp8_gemm_set_attributes();
   if (e == cudaSuccess) e = asap::route_fused_set_attributes();
   if (e != cudaSuccess) return bail(cuda_fail(e, "GEMM attributes"));

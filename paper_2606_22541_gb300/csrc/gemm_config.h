@@ -23,21 +23,18 @@
 #ifndef ASAP_RING_DN_B
 #define ASAP_RING_DN_B 4
 #endif
-// paired m-tiles (two 128-row m-tiles per tile sharing the weight boxes): A
-// stages of 2 x 128 rows (32 KB) and B boxes of 32 KB, 3 + 3 stages.
+// paired m-tiles (two 128-row m-tiles per tile sharing the weight boxes; the
+// down GEMM with the fused combine): A stages of 2 x 128 rows (32 KB) and B
+// boxes of 32 KB, 3 + 3 stages.
 #ifndef ASAP_RING_PAIR_A
 #define ASAP_RING_PAIR_A 3
 #endif
 #ifndef ASAP_RING_PAIR_B
 #define ASAP_RING_PAIR_B 3
 #endif
-// A launch runs paired m-tiles when it has at least this many waves of them
-// (estimated, one tile per SM per wave).  Measured on a GB300 against single
-// m-tiles: paired tiles (with half tiles for segment tails) win the gate/up
-// GEMM at every measured size (DeepSeek-V3 4096 tokens 2.40 vs 2.45 ms,
-// Mixtral 1024 tokens 0.44 vs 0.46 ms) and the down GEMM from about three
-// waves (Mixtral 4096 tokens, 3.8 waves: 0.61 vs 0.71 ms), but lose the
-// Mixtral down GEMM at 2.9 waves and below (3072 tokens 0.56 vs 0.53 ms).
+// The down GEMM with the fused combine runs paired m-tiles when it has at least
+// this many waves of them (estimated, one tile per SM per wave): with fewer
+// the larger tile rounds the launch to whole waves more coarsely than it saves.
 #ifndef ASAP_PAIR_MIN_WAVES
 #define ASAP_PAIR_MIN_WAVES 3
 #endif
@@ -46,6 +43,16 @@
 #endif
 #ifndef ASAP_RING_RT_B
 #define ASAP_RING_RT_B 3
+#endif
+
+// CTA pairs: weight and token stages of 16 KB per CTA, 13 in all.  Measured
+// (gate/up us at 4096 / 8192 / 16384 DeepSeek-V3 tokens): 8 + 5 2339 / 3171 /
+// 5746, 7 + 6 2323 / 3122 / 5642, 6 + 7 2309 / 3185 / 5641.
+#ifndef ASAP_RING_CTA2_W
+#define ASAP_RING_CTA2_W 7
+#endif
+#ifndef ASAP_RING_CTA2_X
+#define ASAP_RING_CTA2_X 6
 #endif
 
 // L2 priority of the grouped GEMMs' loads (0 normal, 1 evict-first, 2

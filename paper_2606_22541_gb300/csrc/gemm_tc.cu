@@ -7,6 +7,10 @@
 // list is derived on the device from those offsets, so the host never reads
 // the per-expert counts back (the bubble-free principle of Section 3.4.2).
 //
+// This is the single-CTA form: the router's logits, launches with few rows per
+// expert (bound by the weight stream) and the fused combine; the other expert
+// launches run on CTA pairs (gemm_pair.cu).
+//
 // Design (one CTA per SM, persistent, warp-specialised; 224 threads, 352 with
 // paired m-tiles):
 //   warp 0   : weight producer.  B boxes [256 rows, 64 K] into its ring; the
@@ -21,7 +25,7 @@
 //              paired tile).
 //   epilogue : warps 2-5 (2-9 paired).  tcgen05.ld 32x32b (warp w reads TMEM
 //              lanes 32*(w%4) ...), fused SwiGLU (gate and up columns of a
-//              tile are the two 128-column halves), bf16 stores staged through
+//              tile alternate in eights), bf16 stores staged through
 //              shared memory so each store writes whole 128-byte row pieces
 //              (fp32 router logits are stored directly).
 // Weights: the B descriptors come from the layer table (one entry per layer,
@@ -136,29 +140,34 @@ __device__ __forceinline__ void store_round(const uint32_t* pk, uint4* stage, in
   __syncwarp();
 }
 
-// TMEM -> packed bf16 for 64 output columns starting at output column c0:
-// SwiGLU tiles read gate columns c0 .. c0 + 63 and the matching up columns
-// BN / 2 further and form silu(g) u; plain tiles read columns c0 .. c0 + 63.
-// (16 columns per TMEM wait: 32 or 64 per wait measured the same.)
+// TMEM -> packed bf16 for 64 output columns starting at output column c0.
+// SwiGLU tiles hold gate and up columns alternating in eights (output columns
+// 8j .. 8j + 7: gate at accumulator columns 16j .., up at 16j + 8 ..) and form
+// silu(g) u; plain tiles read columns c0 .. c0 + 63.  (16 columns per TMEM
+// wait for plain tiles: 32 or 64 per wait measured the same.)
 template <int EPI>
 __device__ __forceinline__ void tmem_to_bf16_64(uint32_t taddr, int c0, uint32_t* pk) {
+  if constexpr (EPI == EPI_SWIGLU) {
 #pragma unroll
-  for (int c = 0; c < 64; c += 16) {
-    uint32_t g[16];
-    tmem_ld16(taddr + c0 + c, g);
-    if constexpr (EPI == EPI_SWIGLU) {
-      uint32_t u[16];
-      tmem_ld16(taddr + BN / 2 + c0 + c, u);
+    for (int c = 0; c < 64; c += 16) {
+      uint32_t v[32];
+      tmem_ld32(taddr + 2 * (c0 + c), v);
       tmem_ld_wait();
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        const float g0 = __uint_as_float(g[2 * i]), g1 = __uint_as_float(g[2 * i + 1]);
-        const float u0 = __uint_as_float(u[2 * i]), u1 = __uint_as_float(u[2 * i + 1]);
+        const int j = (i / 4) * 16 + 2 * (i % 4);
+        const float g0 = __uint_as_float(v[j]), g1 = __uint_as_float(v[j + 1]);
+        const float u0 = __uint_as_float(v[j + 8]), u1 = __uint_as_float(v[j + 9]);
         // silu(g) u with the fast exponential and divide (within a few
         // fp32 ulp, far below h's bf16 rounding)
         pk[c / 2 + i] = pack_bf16x2(__fdividef(g0, 1.0f + __expf(-g0)) * u0, __fdividef(g1, 1.0f + __expf(-g1)) * u1);
       }
-    } else {
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 64; c += 16) {
+      uint32_t g[16];
+      tmem_ld16(taddr + c0 + c, g);
       tmem_ld_wait();
 #pragma unroll
       for (int i = 0; i < 8; ++i) pk[c / 2 + i] = pack_bf16x2(__uint_as_float(g[2 * i]), __uint_as_float(g[2 * i + 1]));
@@ -657,9 +666,7 @@ static_assert(sizeof(Sched) + 0 <= 8192, "schedule table");
 
 cudaError_t gemm_set_attributes() {
   cudaError_t e = set_attr<EPI_SWIGLU, false>();
-  if (e == cudaSuccess) e = set_attr<EPI_SWIGLU, true>();
   if (e == cudaSuccess) e = set_attr<EPI_BF16, false>();
-  if (e == cudaSuccess) e = set_attr<EPI_BF16, true>();
   if (e == cudaSuccess) e = set_attr<EPI_BF16, false, true>();
   if (e == cudaSuccess) e = set_attr<EPI_BF16, true, true>();
   if (e == cudaSuccess) e = set_attr<EPI_F32, false>();
@@ -669,20 +676,16 @@ cudaError_t gemm_set_attributes() {
 cudaError_t gemm_launch(int epi, bool pair, const CUtensorMap* maps, const GemmArgs& args, int grid,
                         cudaStream_t stream) {
   if (grid <= 0) return cudaSuccess;
+  // paired m-tiles: the down GEMM with the fused combine only (gemm_pair.cu
+  // runs the other launches of that size)
+  if (pair && !(epi == EPI_BF16 && args.comb_cnt)) return cudaErrorInvalidValue;
   if (epi == EPI_SWIGLU) {
-    if (pair) launch<EPI_SWIGLU, true>(maps, args, grid, stream);
-    else launch<EPI_SWIGLU, false>(maps, args, grid, stream);
+    launch<EPI_SWIGLU, false>(maps, args, grid, stream);
   } else if (epi == EPI_BF16) {
-    if (args.comb_cnt) {
-      if (pair) launch<EPI_BF16, true, true>(maps, args, grid, stream);
-      else launch<EPI_BF16, false, true>(maps, args, grid, stream);
-    } else if (pair) {
-      launch<EPI_BF16, true>(maps, args, grid, stream);
-    } else {
-      launch<EPI_BF16, false>(maps, args, grid, stream);
-    }
+    if (!args.comb_cnt) launch<EPI_BF16, false>(maps, args, grid, stream);
+    else if (pair) launch<EPI_BF16, true, true>(maps, args, grid, stream);
+    else launch<EPI_BF16, false, true>(maps, args, grid, stream);
   } else {
-    if (pair) return cudaErrorInvalidValue;
     launch<EPI_F32, false>(maps, args, grid, stream);
   }
   return cudaGetLastError();

@@ -25,11 +25,13 @@ enum { EPI_SWIGLU = 0, EPI_BF16 = 1, EPI_F32 = 2 };
 // the kernel loads from device memory when it runs.  The entry holds the TMA
 // descriptors of that layer's packed weights (the pre-computed addresses) and
 // plain pointers for what is not read by TMA.
-enum { MAP_ROUTER = 0, MAP_GATE_UP = 1, MAP_DOWN = 2, MAP_SH_GATE_UP = 3, MAP_SH_DOWN = 4, kLayerMaps = 5 };
+// (MAP_PAIR + MAP_*: the expert matrices again, for boxes of 128 rows.)
+enum { MAP_ROUTER = 0, MAP_GATE_UP = 1, MAP_DOWN = 2, MAP_SH_GATE_UP = 3, MAP_SH_DOWN = 4, kLayerMats = 5,
+       MAP_PAIR = 4, kLayerMaps = 9 };
 
 struct alignas(128) LayerEntry {
   CUtensorMap map[kLayerMaps];     // indexed by MAP_*; unused maps are zero
-  const float* scale[kLayerMaps];  // FP8 block scales of the same matrices, else nullptr
+  const float* scale[kLayerMats];  // FP8 block scales of the matrices (MAP_*), else nullptr
   const void* router_w;            // [E, H] bf16
   const float* router_bias;        // [E] fp32 or nullptr
 };
@@ -89,6 +91,11 @@ cudaError_t gemm_set_attributes();
 // sharing the weight boxes (EPI_SWIGLU and EPI_BF16).
 cudaError_t gemm_launch(int epi, bool pair, const CUtensorMap* maps, const GemmArgs& args, int grid,
                         cudaStream_t stream);
+// The same GEMM on CTA pairs (gemm_pair.cu; EPI_SWIGLU, EPI_BF16, problem 0
+// with offsets): maps A0 for boxes of 32, 64, 96 and 128 rows, A1 likewise, O0, O1
+// (boxes of 32 rows); args.bmap* are MAP_PAIR + MAP_*.
+cudaError_t pair_gemm_set_attributes();
+cudaError_t pair_gemm_launch(int epi, const CUtensorMap* maps, const GemmArgs& args, int pairs, cudaStream_t stream);
 // Encode a 2-D row-major bf16 tensor [rows, cols] for 128-byte-swizzled
 // boxes of [box_rows, 64].  Returns false and fills *err on failure.
 bool encode_tmap_bf16(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t cols,
@@ -230,12 +237,13 @@ cudaError_t launch_dispatch_fp8_seg(const void* x, int n, int H, int k, int E, c
                                     cudaStream_t s);
 // Expert weights in tile-contiguous order for the grouped GEMMs' weight
 // boxes: box (e, nt, kb) = rows nt*256 .. nt*256+255 of expert e's packed
-// matrix ([E][R] rows of row_bytes; gate_up: packed row nt*256 + r is gate
-// row nt*128 + r for r < 128, else up row nt*128 + r - 128, a = gate, b = up),
+// matrix ([E][R] rows of row_bytes; gate_up: gate (a) and up (b) rows
+// alternate in groups of unit = 1 << log_unit, packed row nt*256 + 2*unit*g + q being gate row
+// nt*128 + unit*g + q for q < unit, else up row nt*128 + unit*g + q - unit),
 // bytes [kb*128, kb*128+128) of each row, stored as 256 consecutive 128-byte
 // rows.  R % 256 == 0 and row_bytes % 128 == 0.
-cudaError_t launch_retile(const void* a, const void* b, int E, int R, long long row_bytes, bool gate_up, void* dst,
-                          cudaStream_t s);
+cudaError_t launch_retile(const void* a, const void* b, int E, int R, long long row_bytes, bool gate_up, int log_unit,
+                          void* dst, cudaStream_t s);
 
 // ------------------------------------------------------------ mailbox
 // The single-GPU form of ASAP's asynchronous dispatch and combine (Sections

@@ -1,0 +1,279 @@
+// Device helpers of the CTA-pair grouped GEMMs: thread-block cluster
+// addressing, cluster-scope mbarriers, the two-SM forms of TMA and tcgen05,
+// fragment-shaped TMEM loads, transposing shared-memory stores, the tile
+// queue shared by the two CTAs and the token-tile schedule.
+//
+// A pair is a cluster of two CTAs on the two SMs of one TPC.  Its tensor cores
+// work on one tile together (tcgen05 cta_group::2): weights are the M operand
+// (256 rows, 128 in each CTA's shared memory and TMEM lanes), tokens the N
+// operand (N rows, N / 2 in each CTA's shared memory), so both operands of an
+// MMA are read from shared memory once per SM instead of the N operand twice.
+#pragma once
+
+#include "common.cuh"
+#include "gemm_sched.cuh"
+#include "internal.h"
+
+namespace asap {
+
+constexpr int kPairRows = 256;     // token rows of a tile at most (N of the MMA)
+constexpr int kPairRowUnit = 32;   // tile heights are multiples of this (N % 32 == 0)
+constexpr uint16_t kPairMask = 3;  // both CTAs of the cluster
+
+// ---------------------------------------------------------------- cluster
+__device__ __forceinline__ uint32_t pair_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// Address, in the cluster's shared window, of this CTA's offset ``addr`` in CTA ``rank``.
+__device__ __forceinline__ uint32_t pair_map(uint32_t addr, uint32_t rank) {
+  uint32_t d;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(rank));
+  return d;
+}
+__device__ __forceinline__ void pair_sync() {
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ void st_pair_u32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+// Arrive on a barrier of either CTA (addr from pair_map).
+__device__ __forceinline__ void mbar_arrive_pair(uint32_t addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+__device__ __forceinline__ bool mbar_try_wait_pair(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// Bounded like mbar_wait, for barriers that the other CTA arrives on.
+__device__ __forceinline__ bool mbar_wait_pair(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  if (mbar_try_wait_pair(bar, parity)) return true;
+  const uint64_t t0 = globaltimer_ns();
+  for (uint32_t i = 1;; ++i) {
+    if (mbar_try_wait_pair(bar, parity)) return true;
+    if ((i & 63u) == 0) {
+      if (*abort_flag) return false;
+      if (globaltimer_ns() - t0 > kWaitLimitNs) return false;
+    }
+  }
+}
+// After a failed wait: copies this thread issued complete on a barrier of the
+// other CTA, which it cannot wait on, so it lets 2 ms pass (a TMA load takes
+// microseconds) before the CTA may wind down.
+__device__ __forceinline__ void drain_delay() {
+  const uint64_t t0 = globaltimer_ns();
+  while (globaltimer_ns() - t0 < 2000000ull) {
+  }
+}
+
+// ---------------------------------------------------------------- rings
+// Position in a ring of N barriers (8 bytes apart from ``bar``): stage s of
+// lap parity ``phase``.
+template <int N>
+struct Ring {
+  int s = 0;
+  uint32_t phase = 0;
+  __device__ __forceinline__ void advance() {
+    if (++s == N) {
+      s = 0;
+      phase ^= 1u;
+    }
+  }
+};
+
+// ---------------------------------------------------------------- two-SM TMA / tcgen05
+// tma_load_2d into this CTA's shared memory, completing on a barrier of either
+// CTA of the pair (bar from pair_map).
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* m, uint32_t bar, int x, int y,
+                                                 uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%3, %4}], [%2], %5;" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(x), "r"(y), "l"(policy)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_alloc_pair(uint32_t dst_smem, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols)
+               : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+// Arrive once on the barrier at this offset in both CTAs when every tcgen05 op
+// this thread issued so far is done.
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+      "h"(kPairMask)
+      : "memory");
+}
+__device__ __forceinline__ void tc_mma_bf16_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                                 uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+
+// ---------------------------------------------------------------- fragments
+// 16 TMEM lanes x 64 (32) columns.  Thread t receives, for each group n of 8
+// columns, lane t / 4 at columns 8n + 2 (t % 4), + 1 in r[4n], r[4n + 1] and
+// lane t / 4 + 8 at the same columns in r[4n + 2], r[4n + 3].
+__device__ __forceinline__ void tmem_ld_frag64(uint32_t taddr, uint32_t (&r)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_ld_frag32(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+// Four 8 x 8 matrices of 16-bit values held like the fragments above (thread
+// t: row t / 4, columns 2 (t % 4), + 1), each stored transposed: column i of
+// matrix m becomes 16 contiguous bytes at the address thread 8m + i passes.
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b),
+               "r"(c), "r"(d)
+               : "memory");
+}
+
+// ---------------------------------------------------------------- token tiles
+// The rows of a segment are cut into the fewest tiles of at most kPairRows
+// rows, of equal height up to kPairRowUnit: a tile's MMA time is proportional
+// to its height, and equal tiles keep the weight bytes per MMA cycle (each
+// tile streams the same weight boxes, from L2 after the first) at their lowest.
+__device__ __forceinline__ int pair_mtiles(int rows) { return (rows + kPairRows - 1) / kPairRows; }
+__device__ __forceinline__ int pair_height(int rows, int mt) {
+  const int h = (rows + mt - 1) / mt;
+  return (h + kPairRowUnit - 1) / kPairRowUnit * kPairRowUnit;
+}
+
+struct alignas(16) PairTile {
+  int row, rows;  // first token row, valid rows
+  int n;          // N of the MMAs: rows rounded up to kPairRowUnit
+  int w_tile;     // 256-row weight tile index in the tensor
+  int n_tile;
+  int k_iters;    // 0: no more tiles
+  int group;
+  int p1;
+};
+
+// Tile t: problem 0 groups in order (n-tile, then token tile innermost, so the
+// pairs that run at the same time share a weight tile through L2), then
+// problem 1 likewise.
+__device__ __forceinline__ void pair_decode(int t, const Sched* s, int G, int total0, const GemmArgs& a, PairTile& T) {
+  int r0, m, local, wt0;
+  if (t < total0) {
+    int lo = 0, hi = G;  // largest g with tile_start[g] <= t
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (s->tile_start[mid] <= t) lo = mid; else hi = mid;
+    }
+    local = t - s->tile_start[lo];
+    r0 = s->row_base[lo];
+    m = s->row_base[lo + 1] - r0;
+    wt0 = lo * (a.b_stride0 / kGemmBN);
+    T.group = lo;
+    T.k_iters = a.k_iters0;
+    T.p1 = 0;
+  } else {
+    local = t - total0;
+    r0 = 0;
+    m = s->m1;
+    wt0 = 0;
+    T.group = 0;
+    T.k_iters = a.k_iters1;
+    T.p1 = 1;
+  }
+  const int mt = pair_mtiles(m), h = pair_height(m, mt);
+  const int nt = local / mt, mi = local - nt * mt;
+  T.row = r0 + mi * h;
+  T.rows = max(0, min(h, m - mi * h));
+  T.n = max(kPairRowUnit, (T.rows + kPairRowUnit - 1) / kPairRowUnit * kPairRowUnit);
+  T.n_tile = nt;
+  T.w_tile = wt0 + nt;
+}
+
+// ---------------------------------------------------------------- tile queue
+// The leader's scheduler warp claims tiles, decodes them and writes the
+// descriptions into both CTAs' queues, one tile ahead of the loads; the
+// consumers of both CTAs release a slot on the leader's barrier.  (With every
+// role popping an id and decoding it itself, the id claimed when the loads
+// reached it, a tile change cost the MMA issuer about 3200 cycles.)
+constexpr int kPairQ = 2;
+constexpr int kPairQBytes = kPairQ * (static_cast<int>(sizeof(PairTile)) + 16);
+
+struct PairQueue {
+  uint32_t q0;    // this CTA's queue: descriptions, full and empty barriers
+  uint32_t lead;  // the leader's, in the cluster window
+  uint32_t n = 0;
+
+  __device__ __forceinline__ uint32_t slot() const { return n % kPairQ; }
+  __device__ __forceinline__ uint32_t phase() const { return (n / kPairQ) & 1u; }
+  __device__ __forceinline__ static uint32_t desc(uint32_t b, uint32_t s) { return b + 32u * s; }
+  __device__ __forceinline__ static uint32_t full(uint32_t b, uint32_t s) { return b + 32u * kPairQ + 8u * s; }
+  __device__ __forceinline__ static uint32_t empty(uint32_t b, uint32_t s) { return b + 40u * kPairQ + 8u * s; }
+
+  __device__ __forceinline__ static void store(uint32_t addr, const PairTile& T) {
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(T.row), "r"(T.rows), "r"(T.n),
+                 "r"(T.w_tile)
+                 : "memory");
+    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr + 16), "r"(T.n_tile), "r"(T.k_iters),
+                 "r"(T.group), "r"(T.p1)
+                 : "memory");
+  }
+  // scheduler thread; peer: the other CTA's queue in the cluster window
+  __device__ __forceinline__ bool push(const PairTile& T, uint32_t peer, volatile int* abort_flag) {
+    const uint32_t s = slot();
+    if (!mbar_wait_pair(empty(q0, s), phase() ^ 1u, abort_flag)) return false;
+    store(desc(lead, s), T);
+    store(desc(peer, s), T);
+    mbar_arrive_pair(full(lead, s));
+    mbar_arrive_pair(full(peer, s));
+    ++n;
+    return true;
+  }
+  // any number of threads of a role; the role releases the slot once
+  __device__ __forceinline__ bool pop(PairTile& T, volatile int* abort_flag) const {
+    const uint32_t s = slot();
+    if (!mbar_wait_pair(full(q0, s), phase(), abort_flag)) return false;
+    const uint32_t a = desc(q0, s);
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(T.row), "=r"(T.rows), "=r"(T.n), "=r"(T.w_tile)
+                 : "r"(a)
+                 : "memory");
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(T.n_tile), "=r"(T.k_iters), "=r"(T.group), "=r"(T.p1)
+                 : "r"(a + 16)
+                 : "memory");
+    return true;
+  }
+  __device__ __forceinline__ void release() const { mbar_arrive_pair(empty(lead, slot())); }
+};
+
+}  // namespace asap

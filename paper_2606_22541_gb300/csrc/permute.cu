@@ -385,17 +385,15 @@ __global__ void __launch_bounds__(kCombineWarps * 32)
   }
 }
 
-// packed[e][b*256 + r] = gate[e][b*128 + r] for r < 128, up[e][b*128 + r - 128]
-// otherwise, so one 256-row weight tile holds 128 gate rows and the matching
-// 128 up rows.
 // Tile-contiguous weights: 128-byte row pieces grouped per GEMM box.
 // dst box (e, nt, kb) = 256 consecutive rows of 128 B: rows nt*256 .. of
 // expert e's packed matrix, bytes [kb*128, kb*128 + 128) of each row; one box
-// is one contiguous 32 KB read from HBM.  gate_up: packed row r of tile nt is
-// gate row nt*128 + r (r < 128) or up row nt*128 + r - 128; else row nt*256 + r
-// of a.  R: packed rows per expert; V: 16-byte units per row.
+// is one contiguous 32 KB read from HBM.  gate_up: in a tile, gate (a) and up
+// (b) rows alternate in groups of 1 << log_unit, so one 256-row tile holds 128 gate
+// rows and the matching 128 up rows.  R: packed rows per expert; V: 16-byte
+// units per row.
 __global__ void retile_kernel(const uint4* __restrict__ a, const uint4* __restrict__ b, int E, int R, int V,
-                              bool gate_up, uint4* __restrict__ dst) {
+                              bool gate_up, int log_unit, uint4* __restrict__ dst) {
   const int KB = V / 8, NT = R / 256;
   const long long total = static_cast<long long>(E) * R * V;
   for (long long q = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; q < total;
@@ -410,7 +408,8 @@ __global__ void retile_kernel(const uint4* __restrict__ a, const uint4* __restri
     const long long e = t / NT;
     const uint4* src;
     if (gate_up)
-      src = (r < 128 ? a : b) + (e * (R / 2) + nt * 128 + (r & 127)) * V;
+      src = ((r >> log_unit) & 1 ? b : a) +
+            (e * (R / 2) + nt * 128 + ((r >> (log_unit + 1)) << log_unit) + (r & ((1 << log_unit) - 1))) * V;
     else
       src = a + (e * R + nt * 256 + r) * V;
     dst[q] = src[kb * 8 + v8];
@@ -511,11 +510,11 @@ cudaError_t launch_combine_mbox(const MboxRound* r, MboxGeom g, const void* y_pe
   return cudaGetLastError();
 }
 
-cudaError_t launch_retile(const void* a, const void* b, int E, int R, long long row_bytes, bool gate_up, void* dst,
-                          cudaStream_t s) {
+cudaError_t launch_retile(const void* a, const void* b, int E, int R, long long row_bytes, bool gate_up, int log_unit,
+                          void* dst, cudaStream_t s) {
   if (R % 256 != 0 || row_bytes % 128 != 0) return cudaErrorInvalidValue;
   retile_kernel<<<4096, 256, 0, s>>>(static_cast<const uint4*>(a), static_cast<const uint4*>(b), E, R,
-                                     static_cast<int>(row_bytes / 16), gate_up, static_cast<uint4*>(dst));
+                                     static_cast<int>(row_bytes / 16), gate_up, log_unit, static_cast<uint4*>(dst));
   return cudaGetLastError();
 }
 
