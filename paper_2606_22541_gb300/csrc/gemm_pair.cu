@@ -312,7 +312,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   pair_sync();  // both CTAs' barriers are initialised
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  PairQueue tq{tq0, pair_map(tq0, 0)};
+  PairQueue tq{tq0, pair_map(tq0, 0), leader};
   // a role that gives up also ends the other CTA's waits
   auto give_up = [&]() {
     *abort_flag = 1;
@@ -365,7 +365,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       ++tq.n;
       if (T.k_iters == 0) break;
       const int acc = it & 1;
-      ok = __all_sync(0xffffffffu, mbar_wait_pair(tempty(acc), ((it >> 1) & 1) ^ 1u, abort_flag));
+      ok = __all_sync(0xffffffffu, mbar_wait(tempty(acc), ((it >> 1) & 1) ^ 1u, abort_flag));
       if (!ok) break;
       tc_fence_after();
       const uint32_t d = tmem_base + acc * 256;

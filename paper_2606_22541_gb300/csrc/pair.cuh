@@ -39,32 +39,24 @@ __device__ __forceinline__ void pair_sync() {
 __device__ __forceinline__ void st_pair_u32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
-// Arrive on a barrier of either CTA (addr from pair_map).
+// Arrive on a barrier of either CTA (addr from pair_map).  Without .cluster
+// scope here and in the waits: what these barriers order is TMEM (fenced by
+// tcgen05) and registers; a cluster-scope release or acquire stalled its thread
+// for 2000 to 4000 cycles behind the loads in flight (tile changes took 300
+// cycles without it; gate/up GEMM of 8192 DeepSeek-V3 tokens 3059 -> 2917 us).
 __device__ __forceinline__ void mbar_arrive_pair(uint32_t addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
 }
-__device__ __forceinline__ bool mbar_try_wait_pair(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
+// Arrive on the other CTA's barrier and expect ``bytes`` of st.async on it.
+__device__ __forceinline__ void mbar_arrive_expect_tx_pair(uint32_t addr, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;" ::"r"(addr), "r"(bytes) : "memory");
 }
-// Bounded like mbar_wait, for barriers that the other CTA arrives on.
-__device__ __forceinline__ bool mbar_wait_pair(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_try_wait_pair(bar, parity)) return true;
-  const uint64_t t0 = globaltimer_ns();
-  for (uint32_t i = 1;; ++i) {
-    if (mbar_try_wait_pair(bar, parity)) return true;
-    if ((i & 63u) == 0) {
-      if (*abort_flag) return false;
-      if (globaltimer_ns() - t0 > kWaitLimitNs) return false;
-    }
-  }
+// 16 bytes into the other CTA's shared memory; its barrier counts them when
+// they are visible there.
+__device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t bar, int a, int b, int c, int d) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%2, %3, %4, %5}, [%1];" ::"r"(addr),
+               "r"(bar), "r"(a), "r"(b), "r"(c), "r"(d)
+               : "memory");
 }
 // After a failed wait: copies this thread issued complete on a barrier of the
 // other CTA, which it cannot wait on, so it lets 2 ms pass (a TMA load takes
@@ -231,6 +223,7 @@ constexpr int kPairQBytes = kPairQ * (static_cast<int>(sizeof(PairTile)) + 16);
 struct PairQueue {
   uint32_t q0;    // this CTA's queue: descriptions, full and empty barriers
   uint32_t lead;  // the leader's, in the cluster window
+  bool leader;    // this CTA is the leader
   uint32_t n = 0;
 
   __device__ __forceinline__ uint32_t slot() const { return n % kPairQ; }
@@ -239,29 +232,27 @@ struct PairQueue {
   __device__ __forceinline__ static uint32_t full(uint32_t b, uint32_t s) { return b + 32u * kPairQ + 8u * s; }
   __device__ __forceinline__ static uint32_t empty(uint32_t b, uint32_t s) { return b + 40u * kPairQ + 8u * s; }
 
-  __device__ __forceinline__ static void store(uint32_t addr, const PairTile& T) {
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(T.row), "r"(T.rows), "r"(T.n),
-                 "r"(T.w_tile)
-                 : "memory");
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr + 16), "r"(T.n_tile), "r"(T.k_iters),
-                 "r"(T.group), "r"(T.p1)
-                 : "memory");
-  }
   // scheduler thread; peer: the other CTA's queue in the cluster window
   __device__ __forceinline__ bool push(const PairTile& T, uint32_t peer, volatile int* abort_flag) {
     const uint32_t s = slot();
-    if (!mbar_wait_pair(empty(q0, s), phase() ^ 1u, abort_flag)) return false;
-    store(desc(lead, s), T);
-    store(desc(peer, s), T);
-    mbar_arrive_pair(full(lead, s));
-    mbar_arrive_pair(full(peer, s));
+    if (!mbar_wait(empty(q0, s), phase() ^ 1u, abort_flag)) return false;
+    const uint32_t pd = desc(peer, s), pb = full(peer, s), ld = desc(q0, s);
+    mbar_arrive_expect_tx_pair(pb, 32);
+    st_async_v4(pd, pb, T.row, T.rows, T.n, T.w_tile);
+    st_async_v4(pd + 16, pb, T.n_tile, T.k_iters, T.group, T.p1);
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ld), "r"(T.row), "r"(T.rows), "r"(T.n), "r"(T.w_tile)
+                 : "memory");
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ld + 16), "r"(T.n_tile), "r"(T.k_iters), "r"(T.group),
+                 "r"(T.p1)
+                 : "memory");
+    mbar_arrive(full(q0, s));
     ++n;
     return true;
   }
   // any number of threads of a role; the role releases the slot once
   __device__ __forceinline__ bool pop(PairTile& T, volatile int* abort_flag) const {
     const uint32_t s = slot();
-    if (!mbar_wait_pair(full(q0, s), phase(), abort_flag)) return false;
+    if (!mbar_wait(full(q0, s), phase(), abort_flag)) return false;
     const uint32_t a = desc(q0, s);
     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
                  : "=r"(T.row), "=r"(T.rows), "=r"(T.n), "=r"(T.w_tile)
@@ -273,7 +264,10 @@ struct PairQueue {
                  : "memory");
     return true;
   }
-  __device__ __forceinline__ void release() const { mbar_arrive_pair(empty(lead, slot())); }
+  __device__ __forceinline__ void release() const {
+    if (leader) mbar_arrive(empty(q0, slot()));
+    else mbar_arrive_pair(empty(lead, slot()));
+  }
 };
 
 }  // namespace asap
