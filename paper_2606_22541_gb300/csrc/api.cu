@@ -522,6 +522,29 @@ int run_expert_ffn(asap_moe_t h, const void* x_perm, const int32_t* offsets, con
   return run_down(h, hbuf, offsets, hsh, n, y_perm, y_sh, layer, counters ? counters + 1 : nullptr, st);
 }
 
+// Launch of an FP8 expert GEMM: e4m3 operands in0 [nk, K0] and in1 [n, K1] (the
+// shared expert's, when f.g.m1 > 0).
+int launch_expert_gemm_fp8(asap_moe_t h, int epi, const void* in0, long long nk, int K0, const void* in1, int n,
+                           int K1, asap::Fp8Args& f, cudaStream_t st) {
+  asap::GemmArgs& a = f.g;
+  const bool sh = a.m1 > 0;
+  std::string err;
+  bool ok = true;
+  constexpr int NB = asap::kFp8Boxes;
+  CUtensorMap maps[2 * NB];
+  for (int i = 0; i < NB; ++i) {
+    ok = ok && asap::encode_tmap_u8(&maps[i], in0, nk, K0, 32 * (i + 1), &err);
+    if (sh) ok = ok && asap::encode_tmap_u8(&maps[NB + i], in1, n, K1, 32 * (i + 1), &err);
+    else maps[NB + i] = maps[i];
+  }
+  if (!ok) return fail(ASAP_ERR_INVALID, "expert GEMM operand: " + err);
+  const long long tiles = static_cast<long long>(ub_mtiles(h->cfg, nk)) * a.n_tiles0 +
+                          (sh ? static_cast<long long>(asap::ceil_div(n, asap::kGemmBM)) * a.n_tiles1 : 0);
+  CU_TRY(asap::fp8_gemm_launch(epi, maps, f, static_cast<int>(std::min<long long>(tiles, h->num_sms)), st),
+         "FP8 expert GEMM launch");
+  return ASAP_OK;
+}
+
 // FP8 GEMM1: hq = e4m3(silu(Xq Wg^T) * (Xq Wu^T)) with its row scales, routed
 // segments plus the shared expert on the quantised x.
 int run_gate_up_fp8(asap_moe_t h, const void* xq, const float* xs, const int32_t* offsets, const void* xq_sh,
@@ -530,15 +553,6 @@ int run_gate_up_fp8(asap_moe_t h, const void* xq, const float* xs, const int32_t
   const asap_moe_config& c = h->cfg;
   const long long nk = static_cast<long long>(n) * c.top_k;
   const bool sh = c.n_shared != 0;
-  std::string err;
-  CUtensorMap maps[2];
-  if (!asap::encode_tmap_u8(&maps[0], xq, nk, c.hidden, asap::kGemmBM, &err)) return fail(ASAP_ERR_INVALID, "x_perm: " + err);
-  if (sh) {
-    if (!asap::encode_tmap_u8(&maps[1], xq_sh, n, c.hidden, asap::kGemmBM, &err))
-      return fail(ASAP_ERR_INVALID, "quantised x: " + err);
-  } else {
-    maps[1] = maps[0];
-  }
   asap::Fp8Args f{};
   asap::GemmArgs& a = f.g;
   a.lref = lref(h, layer);
@@ -574,11 +588,7 @@ int run_gate_up_fp8(asap_moe_t h, const void* xq, const float* xs, const int32_t
   f.o_sld0 = c.inter / 128;
   f.out_scale1 = hs_sh;
   f.o_sld1 = sh ? c.shared_inter / 128 : 0;
-  const long long tiles = static_cast<long long>(ub_mtiles(c, nk)) * a.n_tiles0 +
-                          (sh ? static_cast<long long>(asap::ceil_div(n, asap::kGemmBM)) * a.n_tiles1 : 0);
-  CU_TRY(asap::fp8_gemm_launch(asap::EPI_SWIGLU, maps, f, static_cast<int>(std::min<long long>(tiles, h->num_sms)), st),
-         "fp8 gate/up GEMM launch");
-  return ASAP_OK;
+  return launch_expert_gemm_fp8(h, asap::EPI_SWIGLU, xq, nk, c.hidden, xq_sh, n, c.hidden, f, st);
 }
 
 // FP8 GEMM2: y = (hq * hs) (Wd * sd)^T, bf16 out.
@@ -588,15 +598,6 @@ int run_down_fp8(asap_moe_t h, const void* hq, const float* hs, const int32_t* o
   const asap_moe_config& c = h->cfg;
   const long long nk = static_cast<long long>(n) * c.top_k;
   const bool sh = c.n_shared != 0;
-  std::string err;
-  CUtensorMap maps[2];
-  if (!asap::encode_tmap_u8(&maps[0], hq, nk, c.inter, asap::kGemmBM, &err)) return fail(ASAP_ERR_INVALID, "h: " + err);
-  if (sh) {
-    if (!asap::encode_tmap_u8(&maps[1], hq_sh, n, c.shared_inter, asap::kGemmBM, &err))
-      return fail(ASAP_ERR_INVALID, "h_shared: " + err);
-  } else {
-    maps[1] = maps[0];
-  }
   asap::Fp8Args f{};
   asap::GemmArgs& a = f.g;
   a.lref = lref(h, layer);
@@ -628,11 +629,7 @@ int run_down_fp8(asap_moe_t h, const void* hq, const float* hs, const int32_t* o
   f.a_sld1 = sh ? c.shared_inter / 128 : 0;
   f.b_nblk0 = c.hidden / 128;
   f.b_nblk1 = c.hidden / 128;
-  const long long tiles = static_cast<long long>(ub_mtiles(c, nk)) * a.n_tiles0 +
-                          (sh ? static_cast<long long>(asap::ceil_div(n, asap::kGemmBM)) * a.n_tiles1 : 0);
-  CU_TRY(asap::fp8_gemm_launch(asap::EPI_BF16, maps, f, static_cast<int>(std::min<long long>(tiles, h->num_sms)), st),
-         "fp8 down GEMM launch");
-  return ASAP_OK;
+  return launch_expert_gemm_fp8(h, asap::EPI_BF16, hq, nk, c.inter, hq_sh, n, c.shared_inter, f, st);
 }
 
 }  // namespace
@@ -739,9 +736,9 @@ int pack_layer(asap_moe_t h, const asap_moe_weights* wts, LayerWeights& L, cudaS
       return cuda_fail(e, "copy bias");
   }
   // expert weights in the tile-contiguous order of the GEMMs' weight boxes, so
-  // each box is one 32 KB read; gate/up rows alternate in eights (bf16) or per
-  // 128 rows (FP8)
-  const int log_unit = h->fp8 ? 7 : 3;  // log2 of the rows
+  // each box is one 32 KB read
+  // gate/up rows alternate in eights (bf16) or per 128 rows (FP8)
+  const int log_unit = h->fp8 ? 7 : 3;
   if ((e = cudaMalloc(&L.gate_up, gu_bytes)) != cudaSuccess) return cuda_fail(e, "cudaMalloc gate/up");
   if ((e = asap::launch_retile(wts->w_gate, wts->w_up, static_cast<int>(E), static_cast<int>(2 * I),
                                static_cast<long long>(H * wb), true, log_unit, L.gate_up, st)) != cudaSuccess)

@@ -55,6 +55,14 @@
 #define ASAP_RING_CTA2_X 6
 #endif
 
+// FP8: weight stages of 32 KB, token stages of 16 KB.
+#ifndef ASAP_RING_F8_W
+#define ASAP_RING_F8_W 4
+#endif
+#ifndef ASAP_RING_F8_X
+#define ASAP_RING_F8_X 4
+#endif
+
 // L2 priority of the grouped GEMMs' loads (0 normal, 1 evict-first, 2
 // evict-last): activations (A) are re-read by every n-tile of their expert
 // and stay evict-last; the bf16 weights (B) are read by the m-tiles of one

@@ -277,9 +277,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         args.lref.table[load_layer(args.lref.layer, args.lref.n_layers, args.status, blockIdx.x == 0 && lane == 0)];
     tmW[0] = &le.map[args.bmap0];
     tmW[1] = &le.map[args.bmap1];
+    tensormap_acquire(tmW[0]);
+    if (args.m1 > 0) tensormap_acquire(tmW[1]);
     if (lane == 0) {
-      tensormap_acquire(tmW[0]);
-      if (args.m1 > 0) tensormap_acquire(tmW[1]);
       for (int s = 0; s < SW; ++s) {
         mbar_init(fullW(s), 1);
         mbar_init(emptyW(s), 1);
@@ -332,22 +332,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     }
   } else if (warp == kSchedWarp && lane == 0 && leader) {
     // ------------------------------------------------------------ scheduler
-    const int total0 = sch->tile_start[G];
-    const int total = total0 + pair_mtiles(sch->m1) * args.n_tiles1;
-    const uint32_t peer_q = pair_map(tq0, 1);
-    const int step = static_cast<int>(gridDim.x >> 1);
-    int t = static_cast<int>(blockIdx.x >> 1);
-    PairTile T{};
-    do {
-      const bool more = t < total;
-      if (more) pair_decode(t, sch, G, total0, args, T);
-      else T.k_iters = 0;
-      if (!tq.push(T, peer_q, abort_flag)) {
-        give_up();
-        break;
-      }
-      if (more) t = step + (args.tile_counter ? atomicAdd(args.tile_counter, 1) : t);
-    } while (T.k_iters != 0);
+    if (!pair_schedule<kPairRows>(args, sch, G, tq, pair_map(tq0, 1), abort_flag)) give_up();
   } else if (warp == 1 && leader) {
     // ------------------------------------------------------------ MMA issuer
     // the whole warp runs the loop, one lane issues

@@ -104,9 +104,9 @@ bool encode_tmap_bf16(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t
 // ------------------------------------------------------------ FP8 grouped GEMM
 // e4m3 A and B with fp32 block scales: A scales per row per 128-wide K block
 // ([rows][K/128]), B scales per 128 x 128 block ([groups][N/128][K/128]).
-// Per 128-wide K block the tensor core accumulates into one of two TMEM
-// partial buffers; the epilogue warps add each partial, times the row and
-// block scales, into fp32 registers.
+// Per 128-wide K block the tensor core accumulates into one of the TMEM
+// partials; the epilogue warps add each partial, times the token and block
+// scales, into fp32 registers.
 //  EPI_SWIGLU: out = e4m3 h [rows][N/2] (B rows interleaved 128 gate / 128 up
 //              per 256-row tile, B scale rows interleaved gate / up) and
 //              out_scale = per row per 128 channels of h ([rows][N/256]).
@@ -125,7 +125,10 @@ struct Fp8Args {
 };
 constexpr int kFp8BK = 128;  // K elements (bytes) per stage and per scale block
 
+constexpr int kFp8Boxes = 4;  // A maps of a problem: boxes of 32, 64, 96 and 128 rows
+
 cudaError_t fp8_gemm_set_attributes();
+// maps: A0 and A1 (kFp8Boxes each; A1 may repeat A0 when m1 == 0).
 cudaError_t fp8_gemm_launch(int epi, const CUtensorMap* maps, const Fp8Args& args, int grid, cudaStream_t stream);
 // 2-D row-major byte tensor [rows, cols] for 128-byte-swizzled boxes of [box_rows, 128].
 bool encode_tmap_u8(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows,
@@ -238,10 +241,10 @@ cudaError_t launch_dispatch_fp8_seg(const void* x, int n, int H, int k, int E, c
 // Expert weights in tile-contiguous order for the grouped GEMMs' weight
 // boxes: box (e, nt, kb) = rows nt*256 .. nt*256+255 of expert e's packed
 // matrix ([E][R] rows of row_bytes; gate_up: gate (a) and up (b) rows
-// alternate in groups of unit = 1 << log_unit, packed row nt*256 + 2*unit*g + q being gate row
-// nt*128 + unit*g + q for q < unit, else up row nt*128 + unit*g + q - unit),
-// bytes [kb*128, kb*128+128) of each row, stored as 256 consecutive 128-byte
-// rows.  R % 256 == 0 and row_bytes % 128 == 0.
+// alternate in groups of unit = 1 << log_unit, packed row nt*256 + 2*unit*g + q
+// being gate row nt*128 + unit*g + q for q < unit, else up row nt*128 + unit*g
+// + q - unit), bytes [kb*128, kb*128+128) of each row, stored as 256
+// consecutive 128-byte rows.  R % 256 == 0 and row_bytes % 128 == 0.
 cudaError_t launch_retile(const void* a, const void* b, int E, int R, long long row_bytes, bool gate_up, int log_unit,
                           void* dst, cudaStream_t s);
 

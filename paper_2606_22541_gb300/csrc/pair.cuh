@@ -58,6 +58,11 @@ __device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t bar, int a, 
                "r"(bar), "r"(a), "r"(b), "r"(c), "r"(d)
                : "memory");
 }
+__device__ __forceinline__ void st_async_v2(uint32_t addr, uint32_t bar, uint32_t a, uint32_t b) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%2, %3}, [%1];" ::"r"(addr),
+               "r"(bar), "r"(a), "r"(b)
+               : "memory");
+}
 // After a failed wait: copies this thread issued complete on a barrier of the
 // other CTA, which it cannot wait on, so it lets 2 ms pass (a TMA load takes
 // microseconds) before the CTA may wind down.
@@ -81,6 +86,20 @@ struct Ring {
     }
   }
 };
+
+// The whole warp waits until every lane's barrier (the lanes may look at
+// different ones) has completed its phase.  Bounded like mbar_wait.
+__device__ __forceinline__ bool mbar_wait_all(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  uint64_t t0 = 0;
+  for (uint32_t i = 1;; ++i) {
+    if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
+    if ((i & 255u) == 0) {
+      const uint64_t now = globaltimer_ns();
+      if (t0 == 0) t0 = now;
+      if (__any_sync(0xffffffffu, *abort_flag != 0 || now - t0 > kWaitLimitNs)) return false;
+    }
+  }
+}
 
 // ---------------------------------------------------------------- two-SM TMA / tcgen05
 // tma_load_2d into this CTA's shared memory, completing on a barrier of either
@@ -120,7 +139,7 @@ __device__ __forceinline__ void tc_mma_bf16_pair(uint32_t d_tmem, uint64_t adesc
 }
 
 // ---------------------------------------------------------------- fragments
-// 16 TMEM lanes x 64 (32) columns.  Thread t receives, for each group n of 8
+// 16 TMEM lanes x 64 (32, 16) columns.  Thread t receives, for each group n of 8
 // columns, lane t / 4 at columns 8n + 2 (t % 4), + 1 in r[4n], r[4n + 1] and
 // lane t / 4 + 8 at the same columns in r[4n + 2], r[4n + 3].
 __device__ __forceinline__ void tmem_ld_frag64(uint32_t taddr, uint32_t (&r)[32]) {
@@ -145,6 +164,13 @@ __device__ __forceinline__ void tmem_ld_frag32(uint32_t taddr, uint32_t (&r)[16]
       : "r"(taddr)
       : "memory");
 }
+__device__ __forceinline__ void tmem_ld_frag16(uint32_t taddr, uint32_t (&r)[16]) {  // r[0 .. 7]
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+      : "r"(taddr)
+      : "memory");
+}
 // Four 8 x 8 matrices of 16-bit values held like the fragments above (thread
 // t: row t / 4, columns 2 (t % 4), + 1), each stored transposed: column i of
 // matrix m becomes 16 contiguous bytes at the address thread 8m + i passes.
@@ -155,11 +181,14 @@ __device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, uint32_t a, uin
 }
 
 // ---------------------------------------------------------------- token tiles
-// The rows of a segment are cut into the fewest tiles of at most kPairRows
-// rows, of equal height up to kPairRowUnit: a tile's MMA time is proportional
-// to its height, and equal tiles keep the weight bytes per MMA cycle (each
-// tile streams the same weight boxes, from L2 after the first) at their lowest.
-__device__ __forceinline__ int pair_mtiles(int rows) { return (rows + kPairRows - 1) / kPairRows; }
+// The rows of a segment are cut into the fewest tiles of at most MAXR rows, of
+// equal height up to kPairRowUnit: a tile's MMA time is proportional to its
+// height, and equal tiles keep the weight bytes per MMA cycle (each tile
+// streams the same weight boxes, from L2 after the first) at their lowest.
+template <int MAXR>
+__device__ __forceinline__ int pair_mtiles(int rows) {
+  return (rows + MAXR - 1) / MAXR;
+}
 __device__ __forceinline__ int pair_height(int rows, int mt) {
   const int h = (rows + mt - 1) / mt;
   return (h + kPairRowUnit - 1) / kPairRowUnit * kPairRowUnit;
@@ -178,6 +207,7 @@ struct alignas(16) PairTile {
 // Tile t: problem 0 groups in order (n-tile, then token tile innermost, so the
 // pairs that run at the same time share a weight tile through L2), then
 // problem 1 likewise.
+template <int MAXR>
 __device__ __forceinline__ void pair_decode(int t, const Sched* s, int G, int total0, const GemmArgs& a, PairTile& T) {
   int r0, m, local, wt0;
   if (t < total0) {
@@ -202,7 +232,7 @@ __device__ __forceinline__ void pair_decode(int t, const Sched* s, int G, int to
     T.k_iters = a.k_iters1;
     T.p1 = 1;
   }
-  const int mt = pair_mtiles(m), h = pair_height(m, mt);
+  const int mt = pair_mtiles<MAXR>(m), h = pair_height(m, mt);
   const int nt = local / mt, mi = local - nt * mt;
   T.row = r0 + mi * h;
   T.rows = max(0, min(h, m - mi * h));
@@ -212,9 +242,10 @@ __device__ __forceinline__ void pair_decode(int t, const Sched* s, int G, int to
 }
 
 // ---------------------------------------------------------------- tile queue
-// The leader's scheduler warp claims tiles, decodes them and writes the
-// descriptions into both CTAs' queues, one tile ahead of the loads; the
-// consumers of both CTAs release a slot on the leader's barrier.  (With every
+// One CTA of the pair is the queue's home: its scheduler thread claims tiles,
+// decodes them and writes the descriptions into both CTAs' queues, one tile
+// ahead of the loads; the consumers of both CTAs release a slot on the home's
+// barrier.  (With every
 // role popping an id and decoding it itself, the id claimed when the loads
 // reached it, a tile change cost the MMA issuer about 3200 cycles.)
 constexpr int kPairQ = 2;
@@ -222,8 +253,8 @@ constexpr int kPairQBytes = kPairQ * (static_cast<int>(sizeof(PairTile)) + 16);
 
 struct PairQueue {
   uint32_t q0;    // this CTA's queue: descriptions, full and empty barriers
-  uint32_t lead;  // the leader's, in the cluster window
-  bool leader;    // this CTA is the leader
+  uint32_t home;  // the home's, in the cluster window
+  bool at_home;   // this CTA is the home
   uint32_t n = 0;
 
   __device__ __forceinline__ uint32_t slot() const { return n % kPairQ; }
@@ -232,6 +263,14 @@ struct PairQueue {
   __device__ __forceinline__ static uint32_t full(uint32_t b, uint32_t s) { return b + 32u * kPairQ + 8u * s; }
   __device__ __forceinline__ static uint32_t empty(uint32_t b, uint32_t s) { return b + 40u * kPairQ + 8u * s; }
 
+  __device__ __forceinline__ static void store_local(uint32_t addr, const PairTile& T) {
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(T.row), "r"(T.rows), "r"(T.n),
+                 "r"(T.w_tile)
+                 : "memory");
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr + 16), "r"(T.n_tile), "r"(T.k_iters),
+                 "r"(T.group), "r"(T.p1)
+                 : "memory");
+  }
   // scheduler thread; peer: the other CTA's queue in the cluster window
   __device__ __forceinline__ bool push(const PairTile& T, uint32_t peer, volatile int* abort_flag) {
     const uint32_t s = slot();
@@ -240,11 +279,7 @@ struct PairQueue {
     mbar_arrive_expect_tx_pair(pb, 32);
     st_async_v4(pd, pb, T.row, T.rows, T.n, T.w_tile);
     st_async_v4(pd + 16, pb, T.n_tile, T.k_iters, T.group, T.p1);
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ld), "r"(T.row), "r"(T.rows), "r"(T.n), "r"(T.w_tile)
-                 : "memory");
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ld + 16), "r"(T.n_tile), "r"(T.k_iters), "r"(T.group),
-                 "r"(T.p1)
-                 : "memory");
+    store_local(ld, T);
     mbar_arrive(full(q0, s));
     ++n;
     return true;
@@ -265,9 +300,51 @@ struct PairQueue {
     return true;
   }
   __device__ __forceinline__ void release() const {
-    if (leader) mbar_arrive(empty(q0, slot()));
-    else mbar_arrive_pair(empty(lead, slot()));
+    if (at_home) mbar_arrive(empty(q0, slot()));
+    else mbar_arrive_pair(empty(home, slot()));
   }
 };
+
+// The same queue within one CTA (home and only consumer).
+__device__ __forceinline__ bool local_push(PairQueue& tq, const PairTile& T, volatile int* abort_flag) {
+  const uint32_t s = tq.slot();
+  if (!mbar_wait(PairQueue::empty(tq.q0, s), tq.phase() ^ 1u, abort_flag)) return false;
+  PairQueue::store_local(PairQueue::desc(tq.q0, s), T);
+  mbar_arrive(PairQueue::full(tq.q0, s));
+  ++tq.n;
+  return true;
+}
+
+// The scheduler thread: claims and decodes this worker's tiles (worker: a CTA or
+// a pair; the first tile is its index, the next ones come from the launch's
+// counter) and pushes them.  Returns false when a wait ran out.
+template <int MAXR, typename Push>
+__device__ __forceinline__ bool feed_tiles(const GemmArgs& args, const Sched* sch, int G, int worker, int workers,
+                                           Push push) {
+  const int total0 = sch->tile_start[G];
+  const int total = total0 + pair_mtiles<MAXR>(sch->m1) * args.n_tiles1;
+  int t = worker;
+  PairTile T{};
+  do {
+    const bool more = t < total;
+    if (more) pair_decode<MAXR>(t, sch, G, total0, args, T);
+    else T.k_iters = 0;
+    if (!push(T)) return false;
+    if (more) t = workers + (args.tile_counter ? atomicAdd(args.tile_counter, 1) : t);
+  } while (T.k_iters != 0);
+  return true;
+}
+template <int MAXR>
+__device__ __forceinline__ bool pair_schedule(const GemmArgs& args, const Sched* sch, int G, PairQueue& tq,
+                                              uint32_t peer, volatile int* abort_flag) {
+  return feed_tiles<MAXR>(args, sch, G, static_cast<int>(blockIdx.x >> 1), static_cast<int>(gridDim.x >> 1),
+                          [&](const PairTile& T) { return tq.push(T, peer, abort_flag); });
+}
+template <int MAXR>
+__device__ __forceinline__ bool tile_schedule(const GemmArgs& args, const Sched* sch, int G, PairQueue& tq,
+                                              volatile int* abort_flag) {
+  return feed_tiles<MAXR>(args, sch, G, static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x),
+                          [&](const PairTile& T) { return local_push(tq, T, abort_flag); });
+}
 
 }  // namespace asap

@@ -388,10 +388,9 @@ __global__ void __launch_bounds__(kCombineWarps * 32)
 // Tile-contiguous weights: 128-byte row pieces grouped per GEMM box.
 // dst box (e, nt, kb) = 256 consecutive rows of 128 B: rows nt*256 .. of
 // expert e's packed matrix, bytes [kb*128, kb*128 + 128) of each row; one box
-// is one contiguous 32 KB read from HBM.  gate_up: in a tile, gate (a) and up
-// (b) rows alternate in groups of 1 << log_unit, so one 256-row tile holds 128 gate
-// rows and the matching 128 up rows.  R: packed rows per expert; V: 16-byte
-// units per row.
+// is one contiguous 32 KB read from HBM.  A gate/up tile holds 128 gate (a) and
+// the matching 128 up (b) rows, alternating in groups of 1 << log_unit rows.
+// R: packed rows per expert; V: 16-byte units per row.
 __global__ void retile_kernel(const uint4* __restrict__ a, const uint4* __restrict__ b, int E, int R, int V,
                               bool gate_up, int log_unit, uint4* __restrict__ dst) {
   const int KB = V / 8, NT = R / 256;
