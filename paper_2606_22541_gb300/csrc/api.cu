@@ -349,6 +349,11 @@ int ub_mtiles(const asap_moe_config& c, long long nk, int bm = asap::kGemmBM) {
 // warp's 32 rows).
 constexpr uint32_t kStoreRows = 32;
 
+// Token tiles of ``rows`` rows whose operand rows fill ASAP_BLOCK_BYTES.
+int block_tiles(int rows, long long row_bytes) {
+  return static_cast<int>(std::max<long long>(1, ASAP_BLOCK_BYTES / (rows * std::max<long long>(row_bytes, 1))));
+}
+
 // Launch of a bf16 expert GEMM: A operands in0 [nk, K0] and in1 [n, K1] (the
 // shared expert's, when a.m1 > 0), outputs a.out0 and a.out1.
 int launch_expert_gemm(asap_moe_t h, int epi, bool cta2, bool pair, const void* in0, long long nk, int K0,
@@ -372,6 +377,8 @@ int launch_expert_gemm(asap_moe_t h, int epi, bool cta2, bool pair, const void* 
     if (!ok) return fail(ASAP_ERR_INVALID, "expert GEMM operand: " + err);
     a.bmap0 += asap::MAP_PAIR;
     a.bmap1 += asap::MAP_PAIR;
+    a.m_block0 = block_tiles(256, K0 * 2ll);
+    a.m_block1 = block_tiles(256, K1 * 2ll);
     const long long tiles = static_cast<long long>(ub_mtiles(h->cfg, nk, 256)) * a.n_tiles0 +
                             (sh ? static_cast<long long>(asap::ceil_div(n, 256)) * a.n_tiles1 : 0);
     CU_TRY(asap::pair_gemm_launch(epi, maps, a, static_cast<int>(std::min<long long>(tiles, h->num_sms / 2)), st),
@@ -538,6 +545,8 @@ int launch_expert_gemm_fp8(asap_moe_t h, int epi, const void* in0, long long nk,
     else maps[NB + i] = maps[i];
   }
   if (!ok) return fail(ASAP_ERR_INVALID, "expert GEMM operand: " + err);
+  a.m_block0 = block_tiles(asap::kGemmBM, K0);
+  a.m_block1 = block_tiles(asap::kGemmBM, K1);
   const long long tiles = static_cast<long long>(ub_mtiles(h->cfg, nk)) * a.n_tiles0 +
                           (sh ? static_cast<long long>(asap::ceil_div(n, asap::kGemmBM)) * a.n_tiles1 : 0);
   CU_TRY(asap::fp8_gemm_launch(epi, maps, f, static_cast<int>(std::min<long long>(tiles, h->num_sms)), st),

@@ -63,6 +63,25 @@
 #define ASAP_RING_F8_X 4
 #endif
 
+// Tile order of the kernels with a scheduler warp.  Tiles of segments (and the
+// shared expert) with several token tiles are tensor-bound, the others wait for
+// the weight stream: bursts of ASAP_MIX_BURST of the former are spread evenly
+// among the latter.  A burst reads few different weight tiles; with bursts of 1
+// to 8 the shared expert's rows and weights were read from HBM again.  Measured
+// (layer, us; Zipf 4096 and 8045 tokens, balanced 4096, FP8 Zipf 4096): one kind
+// after the other 4110 / 5586 / 3731 / 2615; bursts of 8 3920 / 5332 / 3737 /
+// 2538; 32 3846 / 5202 / 3633 / 2470; 128 4100 / 5379 / 3646 / 2487.
+#ifndef ASAP_MIX_BURST
+#define ASAP_MIX_BURST 32
+#endif
+// Inside a segment the n-tiles are walked per block of token tiles whose operand
+// rows fill this much, so that they are read from HBM once (gate/up GEMM of 8045
+// Zipf tokens, whose largest expert has 86 MB of rows: 3458 -> 3308 us; 16 or 64
+// MB within 2 %).
+#ifndef ASAP_BLOCK_BYTES
+#define ASAP_BLOCK_BYTES (32 << 20)
+#endif
+
 // L2 priority of the grouped GEMMs' loads (0 normal, 1 evict-first, 2
 // evict-last): activations (A) are re-read by every n-tile of their expert
 // and stay evict-last; the bf16 weights (B) are read by the m-tiles of one

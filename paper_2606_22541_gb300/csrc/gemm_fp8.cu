@@ -66,7 +66,7 @@ constexpr int kNumBars = 2 * SW + 2 * SX + 2 * kSlots + 2 + 1;
 constexpr int kQOff = (8 * kNumBars + 15) / 16 * 16;
 constexpr int kBarBytes = kQOff + kPairQBytes + 16;
 constexpr size_t kSmem =
-    SW * kWBytes + SX * kXBytes + kEpiWarps * kStageWarpBytes + kBarBytes + kAmaxBytes + sizeof(Sched);
+    SW * kWBytes + SX * kXBytes + kEpiWarps * kStageWarpBytes + kBarBytes + kAmaxBytes + sizeof(MixSched);
 static_assert(kSmem <= 227 * 1024, "shared memory budget");
 // consumers of a tile: the producers, the epilogue warps and the MMA issuer
 constexpr int kQueueConsumers = 2 + kEpiWarps + 1;
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   int* layer_slot = reinterpret_cast<int*>(tmem_slot + 2);
   float* amax_x = reinterpret_cast<float*>(bar_area + kBarBytes);  // [2][2][kRows]
-  Sched* sch = reinterpret_cast<Sched*>(bar_area + kBarBytes + kAmaxBytes);
+  MixSched* sch = reinterpret_cast<MixSched*>(bar_area + kBarBytes + kAmaxBytes);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = args.groups;
@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_alloc(smem_u32(tmem_slot), kTmemCols);
     tmem_relinquish();
   } else if (warp == 3) {
-    build_schedule<kRows>(args, sch, G, lane);
+    build_mix_schedule<kRows>(args, sch, G, lane);
   }
   tc_fence_before();
   __syncthreads();

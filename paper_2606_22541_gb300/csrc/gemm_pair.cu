@@ -48,7 +48,7 @@ constexpr int kStageBuf = 2 * kBoxBytes;
 constexpr int kStageBytes = 2 * kStageBuf;
 constexpr int kNumBars = 2 * SW + 2 * SX + 5;
 constexpr int kBarBytes = (8 * kNumBars + 15) / 16 * 16 + kPairQBytes + 16;
-constexpr size_t kSmem = SW * kWBytes + SX * kXBytes + kStageBytes + kBarBytes + sizeof(Sched);
+constexpr size_t kSmem = SW * kWBytes + SX * kXBytes + kStageBytes + kBarBytes + sizeof(MixSched);
 static_assert(kSmem <= 227 * 1024, "shared memory budget");
 // consumers of a tile: both CTAs' producers and epilogue warps, the MMA issuer
 constexpr int kQueueConsumers = 2 * (2 + kEpiWarps) + 1;
@@ -264,7 +264,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const uint32_t tq0 = bar0 + kQOff;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_area + kQOff + kPairQBytes);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  Sched* sch = reinterpret_cast<Sched*>(bar_area + kBarBytes);
+  MixSched* sch = reinterpret_cast<MixSched*>(bar_area + kBarBytes);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = pair_rank();
@@ -305,7 +305,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   } else if (warp == 1) {
     tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
   } else if (warp == kSchedWarp && leader) {
-    build_schedule<kPairRows>(args, sch, G, lane);
+    build_mix_schedule<kPairRows>(args, sch, G, lane);
   }
   tc_fence_before();
   __syncthreads();

@@ -16,6 +16,16 @@ struct Sched {
   int m1;  // rows of problem 1 in this launch (args.m1, or *args.m1_dev clamped to [0, args.m1])
 };
 
+// The schedule of the kernels with a scheduler warp: the groups with one token
+// tile per n-tile ("cold", in order), then those with several ("hot", in order).
+struct MixSched {
+  int tile_start[kMaxExperts + 1];  // of the i-th group in that order
+  int row_base[kMaxExperts + 1];    // of group g
+  int cold;  // tiles of the cold groups
+  int m1;    // rows of problem 1
+  uint8_t group[kMaxExperts];       // the i-th group
+};
+
 struct Tile {
   int a_row, b_row, rows, n_tile, kb0, kb1, split, group;
   bool p1;
@@ -180,6 +190,76 @@ __device__ __forceinline__ void build_schedule(const GemmArgs& args, Sched* sch,
   if (lane == 31) {
     sch->tile_start[G] = incl;
     sch->row_base[G] = args.offsets ? __ldg(args.offsets + G) : args.m0;
+  }
+}
+
+// MixSched for tiles of at most MAXR rows (one full warp).
+template <int MAXR>
+__device__ __forceinline__ void build_mix_schedule(const GemmArgs& args, MixSched* sch, int G, int lane) {
+  if (lane == 0) sch->m1 = args.m1_dev ? min(max(__ldg(args.m1_dev), 0), args.m1) : args.m1;
+  int lo[8], m[8];
+  bool bad = false;
+  int nc = 0, nh = 0, tc = 0, th = 0;  // this lane's cold / hot groups and tiles
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int g = lane * 8 + i;
+    lo[i] = 0;
+    m[i] = 0;
+    if (g < G) {
+      lo[i] = __ldg(args.offsets + g);
+      const int hi = __ldg(args.offsets + g + 1);
+      m[i] = hi - lo[i];
+      bad |= lo[i] < 0 || m[i] < 0 || hi > args.m0;
+      const int mt = (max(m[i], 0) + MAXR - 1) / MAXR;
+      if (mt <= 1) {
+        ++nc;
+        tc += mt * args.n_tiles0;
+      } else {
+        ++nh;
+        th += mt * args.n_tiles0;
+      }
+    }
+  }
+  if (__any_sync(0xffffffffu, bad)) {
+    if (lane == 0) {
+      record_status(args.status, ST_BAD_OFFSETS);
+      sch->cold = 0;
+    }
+    for (int g = lane; g <= G; g += 32) sch->tile_start[g] = 0;
+    return;
+  }
+  int inc = nc, inh = nh, itc = tc, ith = th;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int a = __shfl_up_sync(0xffffffffu, inc, o), b = __shfl_up_sync(0xffffffffu, inh, o);
+    const int c = __shfl_up_sync(0xffffffffu, itc, o), d = __shfl_up_sync(0xffffffffu, ith, o);
+    if (lane >= o) {
+      inc += a;
+      inh += b;
+      itc += c;
+      ith += d;
+    }
+  }
+  const int cold_groups = __shfl_sync(0xffffffffu, inc, 31), cold = __shfl_sync(0xffffffffu, itc, 31);
+  int pc = inc - nc, ph = cold_groups + inh - nh;  // positions
+  int sc = itc - tc, sh = cold + ith - th;         // first tiles
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int g = lane * 8 + i;
+    if (g < G) {
+      const int mt = (m[i] + MAXR - 1) / MAXR;
+      const int p = mt <= 1 ? pc++ : ph++;
+      int& s = mt <= 1 ? sc : sh;
+      sch->tile_start[p] = s;
+      sch->row_base[g] = lo[i];
+      sch->group[p] = static_cast<uint8_t>(g);
+      s += mt * args.n_tiles0;
+    }
+  }
+  if (lane == 31) {
+    sch->tile_start[G] = cold + ith;
+    sch->row_base[G] = __ldg(args.offsets + G);
+    sch->cold = cold;
   }
 }
 

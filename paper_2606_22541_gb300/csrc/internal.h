@@ -66,6 +66,7 @@ struct GemmArgs {
   LayerRef lref;           // B of problem p is lref.table[layer].map[bmap_p]
   int bmap0, bmap1;
   int* tile_counter;       // zero at launch: tiles are claimed dynamically; nullptr: static order
+  int m_block0, m_block1;  // token tiles per block of the tile order (kernels with a scheduler warp)
   int b_tiled;             // B in tile-contiguous order (launch_retile): box row ((b_row/256) k_iters + kb) 256
   // combine fused into the down GEMM (EPI_BF16 only; comb_cnt == nullptr: off)
   int* comb_cnt;             // [comb_n, n_tiles0] arrivals per token slice, zero at launch

@@ -11,6 +11,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "gemm_config.h"
 #include "gemm_sched.cuh"
 #include "internal.h"
 
@@ -204,27 +205,42 @@ struct alignas(16) PairTile {
   int p1;
 };
 
-// Tile t: problem 0 groups in order (n-tile, then token tile innermost, so the
-// pairs that run at the same time share a weight tile through L2), then
-// problem 1 likewise.
+// Position, in the order cold groups, hot groups, problem 1, of the t-th tile
+// handed out: the tiles from ``cold`` on come in bursts spread evenly over the
+// launch (burst k from tile ceil(k Q total / hot) on).
+__device__ __forceinline__ int mix_position(int t, int cold, int total) {
+  const int hot = total - cold;
+  if (hot == 0) return t;
+  constexpr int Q = ASAP_MIX_BURST;
+  const int k = static_cast<int>(static_cast<long long>(t) * hot / (static_cast<long long>(Q) * total));
+  const int tk = static_cast<int>((static_cast<long long>(k) * Q * total + hot - 1) / hot);
+  if (t >= tk && t - tk < Q && k * Q + t - tk < hot) return cold + k * Q + t - tk;
+  return t - min(t >= tk ? (k + 1) * Q : k * Q, hot);
+}
+
+// The t-th tile of the launch.  Inside a group: block of m_block token tiles,
+// n-tile, then token tile innermost, so the workers that run at the same time
+// share a weight tile through L2 and a block's rows stay in L2 over its n-tiles.
 template <int MAXR>
-__device__ __forceinline__ void pair_decode(int t, const Sched* s, int G, int total0, const GemmArgs& a, PairTile& T) {
+__device__ __forceinline__ void pair_decode(int t, const MixSched* s, int G, int total0, int total, const GemmArgs& a,
+                                            PairTile& T) {
   int r0, m, local, wt0;
-  if (t < total0) {
-    int lo = 0, hi = G;  // largest g with tile_start[g] <= t
+  const int u = mix_position(t, s->cold, total);
+  if (u < total0) {
+    int lo = 0, hi = G;  // largest g with tile_start[g] <= u
     while (hi - lo > 1) {
       const int mid = (lo + hi) >> 1;
-      if (s->tile_start[mid] <= t) lo = mid; else hi = mid;
+      if (s->tile_start[mid] <= u) lo = mid; else hi = mid;
     }
-    local = t - s->tile_start[lo];
-    r0 = s->row_base[lo];
-    m = s->row_base[lo + 1] - r0;
-    wt0 = lo * (a.b_stride0 / kGemmBN);
-    T.group = lo;
+    local = u - s->tile_start[lo];
+    T.group = s->group[lo];
+    r0 = s->row_base[T.group];
+    m = s->row_base[T.group + 1] - r0;
+    wt0 = T.group * (a.b_stride0 / kGemmBN);
     T.k_iters = a.k_iters0;
     T.p1 = 0;
   } else {
-    local = t - total0;
+    local = u - total0;
     r0 = 0;
     m = s->m1;
     wt0 = 0;
@@ -233,7 +249,12 @@ __device__ __forceinline__ void pair_decode(int t, const Sched* s, int G, int to
     T.p1 = 1;
   }
   const int mt = pair_mtiles<MAXR>(m), h = pair_height(m, mt);
-  const int nt = local / mt, mi = local - nt * mt;
+  const int mb = T.p1 ? a.m_block1 : a.m_block0;  // token tiles per block
+  const int per = mb * (T.p1 ? a.n_tiles1 : a.n_tiles0);
+  const int b = local / per;
+  local -= b * per;
+  const int sz = min(mb, mt - b * mb);
+  const int nt = local / sz, mi = b * mb + local - nt * sz;
   T.row = r0 + mi * h;
   T.rows = max(0, min(h, m - mi * h));
   T.n = max(kPairRowUnit, (T.rows + kPairRowUnit - 1) / kPairRowUnit * kPairRowUnit);
@@ -319,7 +340,7 @@ __device__ __forceinline__ bool local_push(PairQueue& tq, const PairTile& T, vol
 // a pair; the first tile is its index, the next ones come from the launch's
 // counter) and pushes them.  Returns false when a wait ran out.
 template <int MAXR, typename Push>
-__device__ __forceinline__ bool feed_tiles(const GemmArgs& args, const Sched* sch, int G, int worker, int workers,
+__device__ __forceinline__ bool feed_tiles(const GemmArgs& args, const MixSched* sch, int G, int worker, int workers,
                                            Push push) {
   const int total0 = sch->tile_start[G];
   const int total = total0 + pair_mtiles<MAXR>(sch->m1) * args.n_tiles1;
@@ -327,7 +348,7 @@ __device__ __forceinline__ bool feed_tiles(const GemmArgs& args, const Sched* sc
   PairTile T{};
   do {
     const bool more = t < total;
-    if (more) pair_decode<MAXR>(t, sch, G, total0, args, T);
+    if (more) pair_decode<MAXR>(t, sch, G, total0, total, args, T);
     else T.k_iters = 0;
     if (!push(T)) return false;
     if (more) t = workers + (args.tile_counter ? atomicAdd(args.tile_counter, 1) : t);
@@ -335,13 +356,13 @@ __device__ __forceinline__ bool feed_tiles(const GemmArgs& args, const Sched* sc
   return true;
 }
 template <int MAXR>
-__device__ __forceinline__ bool pair_schedule(const GemmArgs& args, const Sched* sch, int G, PairQueue& tq,
+__device__ __forceinline__ bool pair_schedule(const GemmArgs& args, const MixSched* sch, int G, PairQueue& tq,
                                               uint32_t peer, volatile int* abort_flag) {
   return feed_tiles<MAXR>(args, sch, G, static_cast<int>(blockIdx.x >> 1), static_cast<int>(gridDim.x >> 1),
                           [&](const PairTile& T) { return tq.push(T, peer, abort_flag); });
 }
 template <int MAXR>
-__device__ __forceinline__ bool tile_schedule(const GemmArgs& args, const Sched* sch, int G, PairQueue& tq,
+__device__ __forceinline__ bool tile_schedule(const GemmArgs& args, const MixSched* sch, int G, PairQueue& tq,
                                               volatile int* abort_flag) {
   return feed_tiles<MAXR>(args, sch, G, static_cast<int>(blockIdx.x), static_cast<int>(gridDim.x),
                           [&](const PairTile& T) { return local_push(tq, T, abort_flag); });

@@ -17,6 +17,7 @@ SEGMENTS = [
     [65, 127, 128, 129, 255, 256, 0, 0],      # up to one full tile
     [257, 289, 511, 512, 513, 0, 7, 1],       # two and three tiles of equal height
     [0, 0, 0, 0, 0, 0, 0, 2],                 # one token
+    [2100, 700, 40, 33, 1, 0, 300, 260],      # bursts of many-tile segments among the others
 ]
 
 
@@ -58,6 +59,32 @@ def test_segments_at_tile_edges(rows, n_shared):
         assert torch.equal(ysh.view(torch.int16), outs[api.TILING_SINGLE][1].view(torch.int16))
         compare_rows(ysh.double().cpu().numpy(),
                      _ffn64(x, w["sh_gate"], w["sh_up"], w["sh_down"]).cpu().numpy())
+    h.close()
+
+
+def test_blocks_of_token_tiles():
+    """A segment whose rows fill more than one block of the tile order (2048
+    rows of 16 KB), beside a short one: every row, bit for bit."""
+    cfg = inputs.small_variant(MIXTRAL, name="blocks", n_experts=2, hidden=8192, inter=256, seed=79)
+    rows, n = [4500, 100], 2300
+    w = inputs.make_weights(cfg, DEV)
+    h = api.asap_moe_create(cfg, w, n)
+    xp = inputs.randn_bf16((2 * n, cfg.hidden), 1.0, 1, DEV)
+    x = inputs.randn_bf16((n, cfg.hidden), 1.0, 2, DEV)
+    offs = torch.tensor([0] + rows, device=DEV).cumsum(0).to(torch.int32)
+    outs = []
+    for mode in (api.TILING_SINGLE, api.TILING_PAIRED):
+        api.asap_moe_set_tiling(h, mode)
+        y = torch.full((2 * n, cfg.hidden), float("nan"), dtype=torch.bfloat16, device=DEV)
+        api.asap_moe_expert_ffn(h, xp, offs, x, y, None, api.workspace(h, n))
+        torch.cuda.synchronize()
+        outs.append(y)
+    assert api.asap_moe_status(h) == (0, 0)
+    assert torch.equal(outs[0].view(torch.int16), outs[1].view(torch.int16))
+    t = torch.tensor([0, 2047, 2048, 4499, 4500, 4599], device=DEV)
+    for e, sel in ((0, t[:4]), (1, t[4:])):
+        compare_rows(outs[1][sel].double().cpu().numpy(),
+                     _ffn64(xp[sel], w["w_gate"][e], w["w_up"][e], w["w_down"][e]).cpu().numpy())
     h.close()
 
 
