@@ -73,35 +73,6 @@ __device__ __forceinline__ void drain_delay() {
   }
 }
 
-// ---------------------------------------------------------------- rings
-// Position in a ring of N barriers (8 bytes apart from ``bar``): stage s of
-// lap parity ``phase``.
-template <int N>
-struct Ring {
-  int s = 0;
-  uint32_t phase = 0;
-  __device__ __forceinline__ void advance() {
-    if (++s == N) {
-      s = 0;
-      phase ^= 1u;
-    }
-  }
-};
-
-// The whole warp waits until every lane's barrier (the lanes may look at
-// different ones) has completed its phase.  Bounded like mbar_wait.
-__device__ __forceinline__ bool mbar_wait_all(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  uint64_t t0 = 0;
-  for (uint32_t i = 1;; ++i) {
-    if (__all_sync(0xffffffffu, mbar_test_wait(bar, parity))) return true;
-    if ((i & 255u) == 0) {
-      const uint64_t now = globaltimer_ns();
-      if (t0 == 0) t0 = now;
-      if (__any_sync(0xffffffffu, *abort_flag != 0 || now - t0 > kWaitLimitNs)) return false;
-    }
-  }
-}
-
 // ---------------------------------------------------------------- two-SM TMA / tcgen05
 // tma_load_2d into this CTA's shared memory, completing on a barrier of either
 // CTA of the pair (bar from pair_map).
