@@ -4,9 +4,10 @@
 //
 // Dispatch is the single-GPU form of the token payload the MoE side receives
 // grouped for its experts (ASAP Section 3.2.1); combine returns each expert's
-// result to its token through the expert IDs (Section 3.2.2).  Both move rows
-// as 16-byte vectors with every lane of a warp on consecutive vectors of the
-// same row, so each warp-wide access is 512 contiguous bytes.
+// result to its token through the expert IDs (Section 3.2.2).  Both run one CTA
+// per token and move rows as 16-byte vectors with every lane of a warp on
+// consecutive vectors of the same row, so each warp-wide access is 512
+// contiguous bytes.
 #include "common.cuh"
 #include "internal.h"
 
@@ -17,31 +18,6 @@ namespace asap {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-// The bf16 dispatch splits a chunk's row copies over two CTAs (every one
-// ranks the chunk's entries, the first writes the permutation), so 4096
-// tokens run 256 CTAs, more than the 152 SMs (measured on GB300: 112 -> 107
-// us; four CTAs per chunk: 111 us); the FP8 dispatch, which also quantises,
-// is faster with one CTA per chunk (85 us vs 100 us).
-#ifndef ASAP_DISPATCH_PARTS
-#define ASAP_DISPATCH_PARTS 2
-#endif
-template <bool FP8>
-__host__ __device__ constexpr int dispatch_parts() { return FP8 ? 1 : ASAP_DISPATCH_PARTS; }
-constexpr int kRankWarps = kChunkTokens * kMaxTopK / 32;  // warps that rank the chunk's entries
-template <bool FP8>
-__host__ __device__ constexpr int dispatch_warps() {
-  return kChunkTokens / dispatch_parts<FP8>() > kRankWarps ? kChunkTokens / dispatch_parts<FP8>() : kRankWarps;
-}
-
-// One CTA per chunk of kChunkTokens tokens.  Entry i = t_local * k + j is
-// ranked by thread i, so warp order and lane order follow (t, j); the rank of
-// an entry inside its expert is (entries of that expert in earlier chunks)
-// + (in earlier warps of this chunk) + (in earlier lanes of this warp):
-// positions increase with (t, j) inside every segment.  chunk_base is
-// chunk-major, relative to the expert's offset: the entries of expert e in
-// chunks before ``chunk`` are offsets[e] + chunk_base[chunk * E + e].
-// Then one warp per token
-// reads its row once and writes it to its k positions.
 // Quantise 8 consecutive values of a 128-channel block held by 16 lanes
 // (lanes 0-15 one block, 16-31 the next): scale = amax / 448 over the block,
 // q = e4m3(v / scale) with round-to-nearest-even and saturation; the
@@ -69,123 +45,118 @@ __device__ __forceinline__ uint2 quantize8(uint4 v, float& scale) {
   return make_uint2(w[0], w[1]);
 }
 
-// Chunk c (part ``part`` of its row copies) of one micro-batch; the body of
-// the dispatch kernels (one CTA per chunk and part).
-template <bool FP8>
-__device__ __forceinline__ void dispatch_chunk(int c, int part, const uint4* __restrict__ x, int n, int V, int k,
-                                               int E, const int32_t* __restrict__ idx,
-                                               const int32_t* __restrict__ chunk_base, void* __restrict__ x_perm_v,
-                                               float* __restrict__ xs, uint2* __restrict__ xq_sh,
-                                               float* __restrict__ xs_sh, int32_t* __restrict__ perm_src,
-                                               int32_t* __restrict__ perm_dst, uint32_t* status,
-                                               const DispatchSeg& seg) {
-  __shared__ int wcnt[kRankWarps][kMaxExperts];
-  __shared__ int spos[kChunkTokens * kMaxTopK];
-  constexpr int kParts = dispatch_parts<FP8>();
-  const int t0 = c * kChunkTokens;
-  const int nt = min(kChunkTokens, n - t0);
-  const int ne = nt * k;
-  const long long nk = seg.rows_total;  // positions of every micro-batch of the call
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < kRankWarps * E; i += blockDim.x) wcnt[i / E][i % E] = 0;
-  __syncthreads();
+// Dispatch: one CTA per token.  The CTA finds the token's k positions and writes
+// its row to them; every thread has its vectors of the row in flight before it
+// looks at the routing, so the chain from idx to a position (expert, chunk base,
+// rank) hides behind the row's load.  Bound by HBM writes (k per row read).
+// Against CTAs of 16 tokens with a warp per token (which ranked the whole chunk
+// and then walked each row with one warp) asap_moe_dispatch took, at 100 / 1024 /
+// 2591 / 4096 / 16384 tokens: 17 / 38 / 66 / 95 / 327 us, 45 / 49 / 91 / 108 / 354
+// before; the FP8 dispatch of a layer call at 1108 / 4096 tokens 19 / 52 us, 52 /
+// 68 before.
+constexpr int kDispatchThreads = 256;
+constexpr int kDispatchAhead = 4;  // vectors of the row per thread in flight
+static_assert(kDispatchThreads == kChunkTokens * kMaxTopK, "one thread per entry of a chunk");
 
-  const int i = threadIdx.x;
-  int e = -1, rank = 0;
-  if (warp < kRankWarps) {
-    if (i < ne) {
-      e = idx[static_cast<long long>(t0) * k + i];
-      if (e < 0 || e >= E) {
-        record_status(status, ST_BAD_EXPERT_INDEX);
-        e = -1;
-      }
-    }
-    const unsigned peers = __match_any_sync(kFull, e);
-    rank = __popc(peers & ((1u << lane) - 1u));
-    if (e >= 0 && lane == __ffs(peers) - 1) wcnt[warp][e] = __popc(peers);
-  }
-  __syncthreads();
-  for (int ee = threadIdx.x; ee < E; ee += blockDim.x) {
-    int run = seg.expert_offsets[ee] + chunk_base[static_cast<long long>(seg.chunk0 + c) * E + ee];
+// Where a token's rows go: its chunk's entries (idx, t_local * k + j) and bases,
+// its own row t_local of the chunk, and the destinations.
+struct DispatchTok {
+  const uint4* x;             // the token's row
+  const int32_t* idx;         // the chunk's entries
+  int tl;                     // token of the chunk
+  const int32_t* base;        // chunk bases of the chunk, per expert
+  const int32_t* offsets;     // first position per expert
+  int32_t* perm_dst;          // the token's k positions
+  int src;                    // perm_src value
+  uint4* x_sh;                // bf16: copy of the row for the shared expert (nullable)
+  uint2* xq_sh;               // FP8: quantised row and scales for the shared expert (nullable)
+  float* xs_sh;
+};
+
+// Position of entry j: offsets[e] + (entries of e in earlier chunks) + (entries
+// of e before it in this chunk), e its expert; positions increase with (t, j)
+// inside every segment.  An expert outside [0, E) is recorded and has none.
+template <bool FP8>
+__device__ __forceinline__ void dispatch_token(const DispatchTok& d, int V, int k, int E, long long nk,
+                                               void* __restrict__ x_perm_v, float* __restrict__ xs,
+                                               int32_t* __restrict__ perm_src, uint32_t* status) {
+  __shared__ int s_e[kMaxTopK], s_cnt[kMaxTopK], s_pos[kMaxTopK];
+  const int tid = threadIdx.x, lane = tid & 31;
+  uint4 a[kDispatchAhead];
 #pragma unroll
-    for (int w = 0; w < kRankWarps; ++w) {
-      const int v = wcnt[w][ee];
-      wcnt[w][ee] = run;
-      run += v;
+  for (int i = 0; i < kDispatchAhead; ++i)
+    if (tid + i * kDispatchThreads < V) a[i] = __ldg(d.x + tid + i * kDispatchThreads);
+  const int first = d.tl * k;  // the token's first entry in the chunk
+  int e = -1, at = 0;          // thread j < k: entry j's expert and its segment's position for this chunk
+  if (tid < k) {
+    e = d.idx[first + tid];
+    if (e < 0 || e >= E) {
+      record_status(status, ST_BAD_EXPERT_INDEX);
+      e = -1;
+    }
+    s_e[tid] = e;
+    s_cnt[tid] = 0;
+  }
+  const int mine = tid < first + k ? d.idx[tid] : -2;
+  if (e >= 0) at = d.offsets[e] + d.base[e];
+  __syncthreads();
+  if ((tid & ~31) < first + k) {
+    for (int j = 0; j < k; ++j) {
+      const unsigned m = __ballot_sync(kFull, mine == s_e[j] && tid < first + j);
+      if (lane == 0 && m) atomicAdd(&s_cnt[j], __popc(m));
     }
   }
   __syncthreads();
-  if (i < ne) {
+  if (tid < k) {
     int pos = -1;
     if (e >= 0) {
-      pos = wcnt[warp][e] + rank;
+      pos = at + s_cnt[tid];
       if (pos < 0 || pos >= nk) {
         record_status(status, ST_BAD_POSITION);
         pos = -1;
       }
     }
-    spos[i] = pos;
-    if (part == 0) {
-      perm_dst[static_cast<long long>(t0) * k + i] = pos;
-      if (pos >= 0) perm_src[pos] = seg.tok0 + t0 + i / k;
-    }
+    s_pos[tid] = pos;
+    d.perm_dst[tid] = pos;
+    if (pos >= 0) perm_src[pos] = d.src;
   }
   __syncthreads();
-  // row copies: one warp per token of this CTA's part, read once, write k times
-  const int tl = part * (kChunkTokens / kParts) + warp;  // token of the chunk
-  if (warp < kChunkTokens / kParts && tl < nt) {
-    const uint4* src = x + static_cast<long long>(t0 + tl) * V;
-    int p[kMaxTopK];
+  int p[kMaxTopK];
 #pragma unroll
-    for (int j = 0; j < kMaxTopK; ++j) p[j] = j < k ? spos[tl * k + j] : -1;
-    if constexpr (!FP8) {
-      uint4* x_perm = static_cast<uint4*>(x_perm_v);
-      // optional copy of the row for the shared expert (calls that serve
-      // several micro-batches gather their tokens into one matrix)
-      uint4* sh = seg.x_sh ? static_cast<uint4*>(seg.x_sh) + static_cast<long long>(t0 + tl) * V : nullptr;
-      int v = lane;
-      for (; v + 32 < V; v += 64) {
-        const uint4 a = __ldg(src + v);
-        const uint4 b = __ldg(src + v + 32);
+  for (int j = 0; j < kMaxTopK; ++j) p[j] = j < k ? s_pos[j] : -1;
+  for (int v0 = tid; v0 < V; v0 += kDispatchAhead * kDispatchThreads) {
+    if (v0 != tid) {
 #pragma unroll
-        for (int j = 0; j < kMaxTopK; ++j)
-          if (p[j] >= 0) {
-            uint4* d = x_perm + static_cast<long long>(p[j]) * V;
-            d[v] = a;
-            d[v + 32] = b;
+      for (int i = 0; i < kDispatchAhead; ++i)
+        if (v0 + i * kDispatchThreads < V) a[i] = __ldg(d.x + v0 + i * kDispatchThreads);
+    }
+#pragma unroll
+    for (int i = 0; i < kDispatchAhead; ++i) {
+      const int v = v0 + i * kDispatchThreads;
+      if (v < V) {  // (V is a multiple of 32: whole warps)
+        if constexpr (!FP8) {
+          uint4* x_perm = static_cast<uint4*>(x_perm_v);
+#pragma unroll
+          for (int j = 0; j < kMaxTopK; ++j)
+            if (p[j] >= 0) x_perm[static_cast<long long>(p[j]) * V + v] = a[i];
+          if (d.x_sh) d.x_sh[v] = a[i];
+        } else {
+          // 8 values -> 8 bytes; one scale per 16 vectors (128 channels)
+          uint2* xq = static_cast<uint2*>(x_perm_v);
+          float scale;
+          const uint2 q = quantize8(a[i], scale);
+          const int nb = V / 16, blk = v >> 4;
+          const bool head = (lane & 15) == 0;
+#pragma unroll
+          for (int j = 0; j < kMaxTopK; ++j)
+            if (p[j] >= 0) {
+              xq[static_cast<long long>(p[j]) * V + v] = q;
+              if (head) xs[static_cast<long long>(p[j]) * nb + blk] = scale;
+            }
+          if (d.xq_sh) {
+            d.xq_sh[v] = q;
+            if (head) d.xs_sh[blk] = scale;
           }
-        if (sh) {
-          sh[v] = a;
-          sh[v + 32] = b;
-        }
-      }
-      for (; v < V; v += 32) {
-        const uint4 a = __ldg(src + v);
-#pragma unroll
-        for (int j = 0; j < kMaxTopK; ++j)
-          if (p[j] >= 0) x_perm[static_cast<long long>(p[j]) * V + v] = a;
-        if (sh) sh[v] = a;
-      }
-    } else {
-      // e4m3 rows: V vectors of 8 values -> V 8-byte words; one scale per 16
-      // vectors (128 channels); a warp covers two blocks per step
-      uint2* xq = static_cast<uint2*>(x_perm_v);
-      const int nb = V / 16;
-      const long long t = t0 + tl;
-      for (int v = lane; v < V; v += 32) {
-        float scale;
-        const uint2 q = quantize8(__ldg(src + v), scale);
-        const int blk = v >> 4;
-        const bool head = (lane & 15) == 0;
-#pragma unroll
-        for (int j = 0; j < kMaxTopK; ++j)
-          if (p[j] >= 0) {
-            xq[static_cast<long long>(p[j]) * V + v] = q;
-            if (head) xs[static_cast<long long>(p[j]) * nb + blk] = scale;
-          }
-        if (xq_sh) {
-          xq_sh[t * V + v] = q;
-          if (head) xs_sh[t * nb + blk] = scale;
         }
       }
     }
@@ -193,75 +164,66 @@ __device__ __forceinline__ void dispatch_chunk(int c, int part, const uint4* __r
 }
 
 template <bool FP8>
-__global__ void __launch_bounds__(dispatch_warps<FP8>() * 32)
-    dispatch_kernel(const uint4* __restrict__ x, int n, int V, int k, int E,
-                    const int32_t* __restrict__ idx, const int32_t* __restrict__ chunk_base, int n_chunks,
-                    void* __restrict__ x_perm_v, float* __restrict__ xs, uint2* __restrict__ xq_sh,
-                    float* __restrict__ xs_sh, int32_t* __restrict__ perm_src,
+__global__ void __launch_bounds__(kDispatchThreads)
+    dispatch_kernel(const uint4* __restrict__ x, int V, int k, int E, const int32_t* __restrict__ idx,
+                    const int32_t* __restrict__ chunk_base, void* __restrict__ x_perm_v, float* __restrict__ xs,
+                    uint2* __restrict__ xq_sh, float* __restrict__ xs_sh, int32_t* __restrict__ perm_src,
                     int32_t* __restrict__ perm_dst, uint32_t* status, const DispatchSeg seg) {
-  constexpr int kParts = dispatch_parts<FP8>();
-  dispatch_chunk<FP8>(blockIdx.x / kParts, blockIdx.x % kParts, x, n, V, k, E, idx, chunk_base, x_perm_v, xs, xq_sh,
-                      xs_sh, perm_src, perm_dst, status, seg);
+  const int t = blockIdx.x, c = t / kChunkTokens;
+  DispatchTok d;
+  d.x = x + static_cast<long long>(t) * V;
+  d.idx = idx + static_cast<long long>(c) * kChunkTokens * k;
+  d.tl = t % kChunkTokens;
+  d.base = chunk_base + static_cast<long long>(seg.chunk0 + c) * E;
+  d.offsets = seg.expert_offsets;
+  d.perm_dst = perm_dst + static_cast<long long>(t) * k;
+  d.src = seg.tok0 + t;
+  d.x_sh = seg.x_sh ? static_cast<uint4*>(seg.x_sh) + static_cast<long long>(t) * V : nullptr;
+  d.xq_sh = xq_sh ? xq_sh + static_cast<long long>(t) * V : nullptr;
+  d.xs_sh = xq_sh ? xs_sh + static_cast<long long>(t) * (V / 16) : nullptr;
+  dispatch_token<FP8>(d, V, k, E, seg.rows_total, x_perm_v, xs, perm_src, status);
 }
 
-// One work item of a mailbox round's dispatch: part ``part`` of the round's
-// chunk vc (see dispatch_mbox_kernel).
-template <bool FP8>
-__device__ __forceinline__ void dispatch_mbox_item(int vc, int part, const MboxRound* __restrict__ r,
-                                                   const MboxGeom& g, const int32_t* __restrict__ rowmap,
-                                                   const int32_t* __restrict__ idx,
-                                                   const int32_t* __restrict__ chunk_base,
-                                                   const int32_t* __restrict__ offsets, void* __restrict__ x_perm_v,
-                                                   float* __restrict__ xs, void* __restrict__ x_sh,
-                                                   float* __restrict__ xs_sh, int32_t* __restrict__ perm_src,
-                                                   int32_t* __restrict__ perm_dst, uint32_t* status) {
-  const int row = rowmap[vc];
-  const int slot = row / g.slot_chunks;
-  const int c = row - slot * g.slot_chunks;
-  const int i = r->index_of[slot];
-  const int n = r->n[i];
-  const long long tok0 = r->tok0[i];
-  const int V = g.H / 8;
-  DispatchSeg seg{};
-  seg.expert_offsets = offsets;
-  seg.chunk0 = slot * g.slot_chunks;
-  seg.n_chunks_total = g.n_slots * g.slot_chunks;
-  seg.tok0 = static_cast<int>(tok0);
-  seg.rows_total = static_cast<long long>(r->n_total) * g.k;
-  uint2* xq_sh = nullptr;
-  float* xs_sh_i = nullptr;
-  if constexpr (FP8) {
-    if (x_sh) {
-      xq_sh = static_cast<uint2*>(x_sh) + tok0 * V;
-      xs_sh_i = xs_sh + tok0 * (V / 16);
-    }
-  } else {
-    seg.x_sh = x_sh ? static_cast<void*>(static_cast<uint4*>(x_sh) + tok0 * V) : nullptr;
+// The claimed post of a round that holds combined token tg.
+__device__ __forceinline__ int mbox_post(const MboxRound* __restrict__ r, int tg) {
+  int lo = 0, hi = r->count;  // the last claimed post starting at or before tg
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (r->tok0[mid] <= tg) lo = mid; else hi = mid;
   }
-  const long long sidx = static_cast<long long>(slot) * g.slot_tokens * g.k;
-  dispatch_chunk<FP8>(c, part, static_cast<const uint4*>(r->x[i]), n, V, g.k, g.E, idx + sidx, chunk_base, x_perm_v,
-                      xs, xq_sh, xs_sh_i, perm_src, perm_dst + sidx, status, seg);
+  return lo;
 }
 
-// Dispatch of a mailbox round: work item q is part q % kParts of the
-// round's chunk q / kParts in the scan's order (the row map lists the claimed
-// posts' histogram rows, post after post); CTA b takes items b, b + gridDim.x,
-// ...  The chunk's post comes at r->tok0[i] in the combined token order, its
-// histogram row and chunk bases are its slot's, its idx / perm_dst entries
-// its slot's region.
+// Dispatch of a mailbox round: CTA b takes the combined tokens b, b + gridDim.x,
+// ...  A token's post comes at r->tok0[i] in the combined order; its histogram
+// rows and chunk bases are its slot's, its idx / perm_dst entries its slot's
+// region.
 template <bool FP8>
-__global__ void __launch_bounds__(dispatch_warps<FP8>() * 32)
-    dispatch_mbox_kernel(const MboxRound* __restrict__ r, const MboxGeom g, const int32_t* __restrict__ rowmap,
-                         const int32_t* __restrict__ idx, const int32_t* __restrict__ chunk_base,
-                         const int32_t* __restrict__ offsets, void* __restrict__ x_perm_v, float* __restrict__ xs,
-                         void* __restrict__ x_sh, float* __restrict__ xs_sh, int32_t* __restrict__ perm_src,
-                         int32_t* __restrict__ perm_dst, uint32_t* status) {
-  constexpr int kParts = dispatch_parts<FP8>();
-  const int items = r->chunks_total * kParts;
-  for (int q = blockIdx.x; q < items; q += gridDim.x) {
-    dispatch_mbox_item<FP8>(q / kParts, q % kParts, r, g, rowmap, idx, chunk_base, offsets, x_perm_v, xs, x_sh,
-                            xs_sh, perm_src, perm_dst, status);
-    __syncthreads();  // the chunk's shared rank tables are rewritten by the next item
+__global__ void __launch_bounds__(kDispatchThreads)
+    dispatch_mbox_kernel(const MboxRound* __restrict__ r, const MboxGeom g, const int32_t* __restrict__ idx,
+                         const int32_t* __restrict__ chunk_base, const int32_t* __restrict__ offsets,
+                         void* __restrict__ x_perm_v, float* __restrict__ xs, void* __restrict__ x_sh,
+                         float* __restrict__ xs_sh, int32_t* __restrict__ perm_src, int32_t* __restrict__ perm_dst,
+                         uint32_t* status) {
+  const int n_total = r->n_total, V = g.H / 8;
+  const long long nk = static_cast<long long>(n_total) * g.k;
+  for (int tg = blockIdx.x; tg < n_total; tg += gridDim.x) {
+    const int i = mbox_post(r, tg), slot = r->slot[i];
+    const int t = tg - r->tok0[i], c = t / kChunkTokens;
+    const int32_t* sidx = idx + static_cast<long long>(slot) * g.slot_tokens * g.k;
+    DispatchTok d;
+    d.x = static_cast<const uint4*>(r->x[i]) + static_cast<long long>(t) * V;
+    d.idx = sidx + static_cast<long long>(c) * kChunkTokens * g.k;
+    d.tl = t % kChunkTokens;
+    d.base = chunk_base + (static_cast<long long>(slot) * g.slot_chunks + c) * g.E;
+    d.offsets = offsets;
+    d.perm_dst = perm_dst + (static_cast<long long>(slot) * g.slot_tokens + t) * g.k;
+    d.src = tg;
+    d.x_sh = !FP8 && x_sh ? static_cast<uint4*>(x_sh) + static_cast<long long>(tg) * V : nullptr;
+    d.xq_sh = FP8 && x_sh ? static_cast<uint2*>(x_sh) + static_cast<long long>(tg) * V : nullptr;
+    d.xs_sh = FP8 && x_sh ? xs_sh + static_cast<long long>(tg) * (V / 16) : nullptr;
+    dispatch_token<FP8>(d, V, g.k, g.E, nk, x_perm_v, xs, perm_src, status);
+    __syncthreads();  // the token's shared tables are rewritten by the next one
   }
 }
 
@@ -280,16 +242,22 @@ __global__ void __launch_bounds__(256) quantize_rows_kernel(const uint4* __restr
   }
 }
 
-constexpr int kCombineWarps = 8;
+constexpr int kCombineThreads = 256;
+constexpr int kCombineCtas = 3;  // per SM (register cap)
 
-// One warp per token: out[t] = sum_j w[t,j] y_perm[perm_dst[t,j]] (+ y_sh[t]),
+// One CTA per token: out[t] = sum_j w[t,j] y_perm[perm_dst[t,j]] (+ y_sh[t]),
 // fp32 fused multiply-adds in slot order, then the shared row, then bf16.
+// Bound by HBM reads (k + 1 rows per token); a thread has two vectors of every
+// row in flight.  Against one warp per token (28 vectors a lane, a serial chain
+// that a small call could not fill the SMs with) the call took, at 100 / 362 /
+// 2591 / 4096 / 16384 tokens: 12 / 17 / 72 / 104 / 362 us, 39 / 43 / 99 / 113 /
+// 378 before.  (4 CTAs per SM without unrolling 14 / 19 / 74 / 104 / 359; 2 CTAs
+// 12 / 21 / 81 / 119 / 422.)
 // The body for one token: w_t, pd_t its k weights and positions, y_sh_t its
 // shared-expert row (nullable), out_t its output row.
 __device__ __forceinline__ void combine_token(const uint4* __restrict__ y_perm, const uint4* __restrict__ y_sh_t,
                                               const float* __restrict__ w_t, const int32_t* __restrict__ pd_t, int V,
-                                              int k, uint4* __restrict__ out_t, uint32_t* status, long long nk,
-                                              int lane) {
+                                              int k, uint4* __restrict__ out_t, uint32_t* status, long long nk) {
   int p[kMaxTopK];
   float wj[kMaxTopK];
 #pragma unroll
@@ -300,13 +268,13 @@ __device__ __forceinline__ void combine_token(const uint4* __restrict__ y_perm, 
       p[j] = pd_t[j];
       wj[j] = w_t[j];
       if (p[j] < 0 || p[j] >= nk) {
-        if (lane == 0) record_status(status, ST_BAD_POSITION);
+        if (threadIdx.x == 0) record_status(status, ST_BAD_POSITION);
         p[j] = -1;
       }
     }
   }
 #pragma unroll 2
-  for (int v = lane; v < V; v += 32) {
+  for (int v = threadIdx.x; v < V; v += kCombineThreads) {
     uint4 yv[kMaxTopK];
 #pragma unroll
     for (int j = 0; j < kMaxTopK; ++j)
@@ -344,44 +312,32 @@ __device__ __forceinline__ void combine_token(const uint4* __restrict__ y_perm, 
   }
 }
 
-__global__ void __launch_bounds__(kCombineWarps * 32)
+__global__ void __launch_bounds__(kCombineThreads, kCombineCtas)
     combine_kernel(const uint4* __restrict__ y_perm, const uint4* __restrict__ y_sh,
-                   const float* __restrict__ w, const int32_t* __restrict__ perm_dst, int n, int V,
+                   const float* __restrict__ w, const int32_t* __restrict__ perm_dst, int V,
                    int k, uint4* __restrict__ out, uint32_t* status, long long nk) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = blockIdx.x * kCombineWarps + warp;
-  if (t >= n) return;
+  const int t = blockIdx.x;
   const long long tk = static_cast<long long>(t) * k, tv = static_cast<long long>(t) * V;
-  combine_token(y_perm, y_sh ? y_sh + tv : nullptr, w + tk, perm_dst + tk, V, k, out + tv, status, nk, lane);
+  combine_token(y_perm, y_sh ? y_sh + tv : nullptr, w + tk, perm_dst + tk, V, k, out + tv, status, nk);
 }
 
-// Combine of a mailbox round: warp w of CTA b combines the tokens
-// (b + j gridDim.x) * kCombineWarps + w of the round's combined token order
-// (the claimed posts one after the other).  A token's post i (the last with
-// r->tok0[i] <= it) writes into its own output; its weights and positions are
-// in its slot's region, its shared-expert row at its place in the combined
-// order.
-__global__ void __launch_bounds__(kCombineWarps * 32)
+// Combine of a mailbox round: CTA b combines the tokens b, b + gridDim.x, ... of
+// the round's combined token order (the claimed posts one after the other).  A
+// token's post writes into its own output; its weights and positions are in its
+// slot's region, its shared-expert row at its place in the combined order.
+__global__ void __launch_bounds__(kCombineThreads, kCombineCtas)
     combine_mbox_kernel(const MboxRound* __restrict__ r, const MboxGeom g, const uint4* __restrict__ y_perm,
                         const uint4* __restrict__ y_sh, const float* __restrict__ w,
                         const int32_t* __restrict__ perm_dst, uint32_t* status) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int n_total = r->n_total, count = r->count;
+  const int n_total = r->n_total;
   const int V = g.H / 8;
   const long long nk = static_cast<long long>(n_total) * g.k;
-  for (int tg = blockIdx.x * kCombineWarps + warp; tg < n_total; tg += gridDim.x * kCombineWarps) {
-    int lo = 0, hi = count;  // the last claimed post starting at or before tg
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (r->tok0[mid] <= tg) lo = mid; else hi = mid;
-    }
-    const int i = lo;
+  for (int tg = blockIdx.x; tg < n_total; tg += gridDim.x) {
+    const int i = mbox_post(r, tg);
     const int t = tg - r->tok0[i];
-    if (t >= r->n[i]) continue;
     const long long tk = (static_cast<long long>(r->slot[i]) * g.slot_tokens + t) * g.k;
-    combine_token(y_perm, y_sh ? y_sh + (static_cast<long long>(r->tok0[i]) + t) * V : nullptr, w + tk,
-                  perm_dst + tk, V, g.k, static_cast<uint4*>(r->out[i]) + static_cast<long long>(t) * V, status, nk,
-                  lane);
+    combine_token(y_perm, y_sh ? y_sh + static_cast<long long>(tg) * V : nullptr, w + tk, perm_dst + tk, V, g.k,
+                  static_cast<uint4*>(r->out[i]) + static_cast<long long>(t) * V, status, nk);
   }
 }
 
@@ -431,10 +387,9 @@ cudaError_t launch_dispatch_seg(const void* x, int n, int H, int k, int E, const
                                 const int32_t* chunk_base, void* x_perm, int32_t* perm_src, int32_t* perm_dst,
                                 uint32_t* status, const DispatchSeg& seg, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int chunks = ceil_div(n, kChunkTokens);
-  dispatch_kernel<false><<<chunks * dispatch_parts<false>(), dispatch_warps<false>() * 32, 0, s>>>(static_cast<const uint4*>(x), n, H / 8, k, E, idx,
-                                                                chunk_base, seg.n_chunks_total, x_perm, nullptr,
-                                                                nullptr, nullptr, perm_src, perm_dst, status, seg);
+  dispatch_kernel<false><<<n, kDispatchThreads, 0, s>>>(static_cast<const uint4*>(x), H / 8, k, E, idx, chunk_base,
+                                                        x_perm, nullptr, nullptr, nullptr, perm_src, perm_dst, status,
+                                                        seg);
   return cudaGetLastError();
 }
 
@@ -455,11 +410,9 @@ cudaError_t launch_dispatch_fp8_seg(const void* x, int n, int H, int k, int E, c
                                     int32_t* perm_src, int32_t* perm_dst, uint32_t* status, const DispatchSeg& seg,
                                     cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  const int chunks = ceil_div(n, kChunkTokens);
-  dispatch_kernel<true><<<chunks * dispatch_parts<true>(), dispatch_warps<true>() * 32, 0, s>>>(static_cast<const uint4*>(x), n, H / 8, k, E, idx,
-                                                               chunk_base, seg.n_chunks_total, xq, xs,
-                                                               static_cast<uint2*>(xq_sh), xs_sh, perm_src, perm_dst,
-                                                               status, seg);
+  dispatch_kernel<true><<<n, kDispatchThreads, 0, s>>>(static_cast<const uint4*>(x), H / 8, k, E, idx, chunk_base, xq,
+                                                       xs, static_cast<uint2*>(xq_sh), xs_sh, perm_src, perm_dst,
+                                                       status, seg);
   return cudaGetLastError();
 }
 
@@ -474,37 +427,33 @@ cudaError_t launch_combine(const void* y_perm, const void* y_shared, const float
                            const int32_t* perm_dst, int n, int H, int k, void* out, uint32_t* status,
                            cudaStream_t s, long long rows_total) {
   if (n <= 0) return cudaSuccess;
-  combine_kernel<<<ceil_div(n, kCombineWarps), kCombineWarps * 32, 0, s>>>(
-      static_cast<const uint4*>(y_perm), static_cast<const uint4*>(y_shared), w, perm_dst, n, H / 8, k,
+  combine_kernel<<<n, kCombineThreads, 0, s>>>(
+      static_cast<const uint4*>(y_perm), static_cast<const uint4*>(y_shared), w, perm_dst, H / 8, k,
       static_cast<uint4*>(out), status, rows_total > 0 ? rows_total : static_cast<long long>(n) * k);
   return cudaGetLastError();
 }
 
-cudaError_t launch_dispatch_mbox(const MboxRound* r, MboxGeom g, const int32_t* rowmap, const int32_t* idx,
-                                 const int32_t* chunk_base, const int32_t* offsets, void* x_perm, int32_t* perm_src,
-                                 int32_t* perm_dst, void* x_sh, uint32_t* status, cudaStream_t s) {
-  const int grid = g.slot_chunks * dispatch_parts<false>();  // one post's work items; more loop
-  dispatch_mbox_kernel<false><<<grid, dispatch_warps<false>() * 32, 0, s>>>(r, g, rowmap, idx, chunk_base, offsets,
-                                                                            x_perm, nullptr, x_sh, nullptr, perm_src,
-                                                                            perm_dst, status);
+cudaError_t launch_dispatch_mbox(const MboxRound* r, MboxGeom g, const int32_t* idx, const int32_t* chunk_base,
+                                 const int32_t* offsets, void* x_perm, int32_t* perm_src, int32_t* perm_dst,
+                                 void* x_sh, uint32_t* status, cudaStream_t s) {
+  // one post's tokens; more loop
+  dispatch_mbox_kernel<false><<<g.slot_tokens, kDispatchThreads, 0, s>>>(r, g, idx, chunk_base, offsets, x_perm, nullptr,
+                                                                         x_sh, nullptr, perm_src, perm_dst, status);
   return cudaGetLastError();
 }
 
-cudaError_t launch_dispatch_fp8_mbox(const MboxRound* r, MboxGeom g, const int32_t* rowmap, const int32_t* idx,
-                                     const int32_t* chunk_base, const int32_t* offsets, void* xq, float* xs,
-                                     void* xq_sh, float* xs_sh, int32_t* perm_src, int32_t* perm_dst,
-                                     uint32_t* status, cudaStream_t s) {
-  const int grid = g.slot_chunks * dispatch_parts<true>();  // one post's work items; more loop
-  dispatch_mbox_kernel<true><<<grid, dispatch_warps<true>() * 32, 0, s>>>(r, g, rowmap, idx, chunk_base, offsets, xq,
-                                                                          xs, xq_sh, xs_sh, perm_src, perm_dst,
-                                                                          status);
+cudaError_t launch_dispatch_fp8_mbox(const MboxRound* r, MboxGeom g, const int32_t* idx, const int32_t* chunk_base,
+                                     const int32_t* offsets, void* xq, float* xs, void* xq_sh, float* xs_sh,
+                                     int32_t* perm_src, int32_t* perm_dst, uint32_t* status, cudaStream_t s) {
+  dispatch_mbox_kernel<true><<<g.slot_tokens, kDispatchThreads, 0, s>>>(r, g, idx, chunk_base, offsets, xq, xs, xq_sh,
+                                                                        xs_sh, perm_src, perm_dst, status);
   return cudaGetLastError();
 }
 
 cudaError_t launch_combine_mbox(const MboxRound* r, MboxGeom g, const void* y_perm, const void* y_shared,
                                 const float* w, const int32_t* perm_dst, uint32_t* status, cudaStream_t s) {
-  const int grid = ceil_div(g.slot_tokens, kCombineWarps);  // one post's tokens; more loop
-  combine_mbox_kernel<<<grid, kCombineWarps * 32, 0, s>>>(r, g, static_cast<const uint4*>(y_perm),
+  // one post's tokens; more loop
+  combine_mbox_kernel<<<g.slot_tokens, kCombineThreads, 0, s>>>(r, g, static_cast<const uint4*>(y_perm),
                                                           static_cast<const uint4*>(y_shared), w, perm_dst, status);
   return cudaGetLastError();
 }
