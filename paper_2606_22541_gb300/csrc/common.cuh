@@ -53,6 +53,17 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // compiler can overlap the scores of one thread.)
 __device__ __forceinline__ float gate_sigmoid(float l) { return __fdividef(1.0f, 1.0f + __expf(-l)); }
 
+// ---------------------------------------------------------------- dependent launches
+// Kernels are launched with programmatic stream serialisation (launch_pdl): a
+// kernel may start while the one before it on the stream still runs.  Every
+// thread calls pdl_wait before it touches global memory; it returns once the
+// kernel before has completed with its writes visible (and, as every kernel
+// waits so, all kernels before that one).  pdl_launch allows the next kernel to
+// start once every CTA has called it or left.  The small kernels call it when
+// their own wait is over, the GEMMs when a CTA has no tiles left.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---------------------------------------------------------------- smem / timers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));

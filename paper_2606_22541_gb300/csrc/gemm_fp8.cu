@@ -200,13 +200,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const CUtensorMap* tmW[2] = {nullptr, nullptr};
 
   if (warp == 0) {
-    const int l = load_layer(args.lref.layer, args.lref.n_layers, args.status, blockIdx.x == 0 && lane == 0);
-    tmW[0] = &args.lref.table[l].map[args.bmap0];
-    tmW[1] = &args.lref.table[l].map[args.bmap1];
-    tensormap_acquire(tmW[0]);
-    if (args.m1 > 0) tensormap_acquire(tmW[1]);
     if (lane == 0) {
-      *layer_slot = l;
       // one arrival (or commit) each, but for the epilogue's: its warps per
       // partial, its threads per exchange
       for (int i = 0; i < kNumBars; ++i)
@@ -217,6 +211,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       *abort_flag = 0;
       fence_barrier_init();
+    }
+    pdl_wait();
+    const int l = load_layer(args.lref.layer, args.lref.n_layers, args.status, blockIdx.x == 0 && lane == 0);
+    tmW[0] = &args.lref.table[l].map[args.bmap0];
+    tmW[1] = &args.lref.table[l].map[args.bmap1];
+    tensormap_acquire(tmW[0]);
+    if (args.m1 > 0) tensormap_acquire(tmW[1]);
+    if (lane == 0) {
+      *layer_slot = l;
       tma_prefetch_desc(tmW[0]);
       if (args.m1 > 0) tma_prefetch_desc(tmW[1]);
     }
@@ -224,8 +227,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_alloc(smem_u32(tmem_slot), kTmemCols);
     tmem_relinquish();
   } else if (warp == 3) {
+    pdl_wait();
     build_mix_schedule<kRows>(args, sch, G, lane);
   }
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -244,7 +249,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!ok && lane == 0) give_up();
     } else if (warp == 3) {
       // ------------------------------------------------------------ scheduler
-      if (lane == 0 && !tile_schedule<kRows>(args, sch, G, tq, abort_flag)) give_up();
+      if (lane == 0) {
+        if (!tile_schedule<kRows>(args, sch, G, tq, abort_flag)) give_up();
+        pdl_launch();  // no tiles left for this CTA
+      }
     } else {
       // ------------------------------------------------------------ MMA issuer
       const bool issuer = elect_one();
@@ -486,11 +494,9 @@ cudaError_t fp8_gemm_launch(int epi, const CUtensorMap* maps, const Fp8Args& arg
   MapsF8 m;
   for (int p = 0; p < 2; ++p)
     for (int i = 0; i < kFp8Boxes; ++i) m.x[p][i] = maps[kFp8Boxes * p + i];
-  if (epi == EPI_SWIGLU)
-    grouped_gemm_fp8_kernel<EPI_SWIGLU><<<grid, kThreads, kSmem, stream>>>(m, args);
-  else
-    grouped_gemm_fp8_kernel<EPI_BF16><<<grid, kThreads, kSmem, stream>>>(m, args);
-  return cudaGetLastError();
+  return epi == EPI_SWIGLU
+             ? launch_pdl(grouped_gemm_fp8_kernel<EPI_SWIGLU>, dim3(grid), dim3(kThreads), kSmem, stream, 1, m, args)
+             : launch_pdl(grouped_gemm_fp8_kernel<EPI_BF16>, dim3(grid), dim3(kThreads), kSmem, stream, 1, m, args);
 }
 
 bool encode_tmap_u8(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows,

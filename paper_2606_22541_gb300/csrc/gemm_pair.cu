@@ -273,12 +273,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   const CUtensorMap* tmW[2] = {nullptr, nullptr};
 
   if (warp == 0) {
-    const LayerEntry& le =
-        args.lref.table[load_layer(args.lref.layer, args.lref.n_layers, args.status, blockIdx.x == 0 && lane == 0)];
-    tmW[0] = &le.map[args.bmap0];
-    tmW[1] = &le.map[args.bmap1];
-    tensormap_acquire(tmW[0]);
-    if (args.m1 > 0) tensormap_acquire(tmW[1]);
     if (lane == 0) {
       for (int s = 0; s < SW; ++s) {
         mbar_init(fullW(s), 1);
@@ -299,14 +293,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       }
       *abort_flag = 0;
       fence_barrier_init();
+    }
+    pdl_wait();
+    const LayerEntry& le =
+        args.lref.table[load_layer(args.lref.layer, args.lref.n_layers, args.status, blockIdx.x == 0 && lane == 0)];
+    tmW[0] = &le.map[args.bmap0];
+    tmW[1] = &le.map[args.bmap1];
+    tensormap_acquire(tmW[0]);
+    if (args.m1 > 0) tensormap_acquire(tmW[1]);
+    if (lane == 0) {
       tma_prefetch_desc(tmW[0]);
       if (args.m1 > 0) tma_prefetch_desc(tmW[1]);
     }
   } else if (warp == 1) {
     tmem_alloc_pair(smem_u32(tmem_slot), kTmemCols);
   } else if (warp == kSchedWarp && leader) {
+    pdl_wait();
     build_mix_schedule<kPairRows>(args, sch, G, lane);
   }
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   pair_sync();  // both CTAs' barriers are initialised
@@ -333,6 +338,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   } else if (warp == kSchedWarp && lane == 0 && leader) {
     // ------------------------------------------------------------ scheduler
     if (!pair_schedule<kPairRows>(args, sch, G, tq, pair_map(tq0, 1), abort_flag)) give_up();
+    pdl_launch();  // no tiles left for this pair
   } else if (warp == 1 && leader) {
     // ------------------------------------------------------------ MMA issuer
     // the whole warp runs the loop, one lane issues
@@ -429,8 +435,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 
 template <int EPI>
 cudaError_t launch(const PairMaps& maps, const GemmArgs& args, int grid, cudaStream_t stream) {
-  pair_gemm_kernel<EPI><<<dim3(grid), dim3(kThreads), kSmem, stream>>>(maps, args);
-  return cudaGetLastError();
+  return launch_pdl(pair_gemm_kernel<EPI>, dim3(grid), dim3(kThreads), kSmem, stream, 1, maps, args);
 }
 
 }  // namespace

@@ -385,12 +385,6 @@ __global__ void __launch_bounds__(Gemm<EPI, PAIR>::kThreads, 1)
 
   if (warp == 0) {
     if (lane == 0) {
-      const LayerEntry& le =
-          args.lref.table[load_layer(args.lref.layer, args.lref.n_layers, args.status, blockIdx.x == 0)];
-      tmB0 = &le.map[args.bmap0];
-      tmB1 = &le.map[args.bmap1];
-      tensormap_acquire(tmB0);
-      if (args.m1 > 0) tensormap_acquire(tmB1);
       for (int s = 0; s < SA; ++s) {
         mbar_init(fullA(s), 1);
         mbar_init(emptyA(s), 1);
@@ -408,9 +402,18 @@ __global__ void __launch_bounds__(Gemm<EPI, PAIR>::kThreads, 1)
       *abort_flag = 0;
       fence_barrier_init();
       tma_prefetch_desc(&tmA0);
+      if (args.m1 > 0) tma_prefetch_desc(&tmA1);
+    }
+    pdl_wait();
+    if (lane == 0) {
+      const LayerEntry& le =
+          args.lref.table[load_layer(args.lref.layer, args.lref.n_layers, args.status, blockIdx.x == 0)];
+      tmB0 = &le.map[args.bmap0];
+      tmB1 = &le.map[args.bmap1];
+      tensormap_acquire(tmB0);
       tma_prefetch_desc(tmB0);
       if (args.m1 > 0) {
-        tma_prefetch_desc(&tmA1);
+        tensormap_acquire(tmB1);
         tma_prefetch_desc(tmB1);
       }
     }
@@ -419,6 +422,7 @@ __global__ void __launch_bounds__(Gemm<EPI, PAIR>::kThreads, 1)
     tmem_alloc(smem_u32(tmem_slot), kTmemCols);
     tmem_relinquish();
   }
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -455,7 +459,10 @@ __global__ void __launch_bounds__(Gemm<EPI, PAIR>::kThreads, 1)
         ok = false;
         break;
       }
-      if (cur < 0) break;
+      if (cur < 0) {
+        if (isB) pdl_launch();  // no tiles left for this CTA
+        break;
+      }
       Tile T;
       decode_tile<BMT>(cur, sch, G, total0, args, T);
       const CUtensorMap* m = isB ? (T.p1 ? tmB1 : tmB0) : (T.p1 ? &tmA1 : &tmA0);
@@ -635,10 +642,9 @@ cudaError_t set_attr() {
 }
 
 template <int EPI, bool PAIR, bool COMB = false>
-void launch(const CUtensorMap* maps, const GemmArgs& args, int grid, cudaStream_t stream) {
-  grouped_gemm_kernel<EPI, PAIR, COMB>
-      <<<dim3(grid), dim3(Gemm<EPI, PAIR>::kThreads), smem_bytes<EPI, PAIR>(), stream>>>(maps[0], maps[1], maps[2],
-                                                                                        maps[3], args);
+cudaError_t launch(const CUtensorMap* maps, const GemmArgs& args, int grid, cudaStream_t stream) {
+  return launch_pdl(grouped_gemm_kernel<EPI, PAIR, COMB>, dim3(grid), dim3(Gemm<EPI, PAIR>::kThreads),
+                    smem_bytes<EPI, PAIR>(), stream, 1, maps[0], maps[1], maps[2], maps[3], args);
 }
 
 using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -679,16 +685,11 @@ cudaError_t gemm_launch(int epi, bool pair, const CUtensorMap* maps, const GemmA
   // paired m-tiles: the down GEMM with the fused combine only (gemm_pair.cu
   // runs the other launches of that size)
   if (pair && !(epi == EPI_BF16 && args.comb_cnt)) return cudaErrorInvalidValue;
-  if (epi == EPI_SWIGLU) {
-    launch<EPI_SWIGLU, false>(maps, args, grid, stream);
-  } else if (epi == EPI_BF16) {
-    if (!args.comb_cnt) launch<EPI_BF16, false>(maps, args, grid, stream);
-    else if (pair) launch<EPI_BF16, true, true>(maps, args, grid, stream);
-    else launch<EPI_BF16, false, true>(maps, args, grid, stream);
-  } else {
-    launch<EPI_F32, false>(maps, args, grid, stream);
-  }
-  return cudaGetLastError();
+  if (epi == EPI_SWIGLU) return launch<EPI_SWIGLU, false>(maps, args, grid, stream);
+  if (epi != EPI_BF16) return launch<EPI_F32, false>(maps, args, grid, stream);
+  if (!args.comb_cnt) return launch<EPI_BF16, false>(maps, args, grid, stream);
+  return pair ? launch<EPI_BF16, true, true>(maps, args, grid, stream)
+              : launch<EPI_BF16, false, true>(maps, args, grid, stream);
 }
 
 bool encode_tmap_bf16(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t cols,

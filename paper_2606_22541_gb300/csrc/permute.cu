@@ -169,6 +169,8 @@ __global__ void __launch_bounds__(kDispatchThreads)
                     const int32_t* __restrict__ chunk_base, void* __restrict__ x_perm_v, float* __restrict__ xs,
                     uint2* __restrict__ xq_sh, float* __restrict__ xs_sh, int32_t* __restrict__ perm_src,
                     int32_t* __restrict__ perm_dst, uint32_t* status, const DispatchSeg seg) {
+  pdl_wait();
+  pdl_launch();
   const int t = blockIdx.x, c = t / kChunkTokens;
   DispatchTok d;
   d.x = x + static_cast<long long>(t) * V;
@@ -205,6 +207,8 @@ __global__ void __launch_bounds__(kDispatchThreads)
                          void* __restrict__ x_perm_v, float* __restrict__ xs, void* __restrict__ x_sh,
                          float* __restrict__ xs_sh, int32_t* __restrict__ perm_src, int32_t* __restrict__ perm_dst,
                          uint32_t* status) {
+  pdl_wait();
+  pdl_launch();
   const int n_total = r->n_total, V = g.H / 8;
   const long long nk = static_cast<long long>(n_total) * g.k;
   for (int tg = blockIdx.x; tg < n_total; tg += gridDim.x) {
@@ -230,6 +234,8 @@ __global__ void __launch_bounds__(kDispatchThreads)
 // Rows of bf16 to e4m3 with a scale per 128 channels; one warp per row.
 __global__ void __launch_bounds__(256) quantize_rows_kernel(const uint4* __restrict__ x, int rows, int V,
                                                             uint2* __restrict__ q, float* __restrict__ s) {
+  pdl_wait();
+  pdl_launch();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long r = static_cast<long long>(blockIdx.x) * 8 + warp;
   if (r >= rows) return;
@@ -316,6 +322,8 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtas)
     combine_kernel(const uint4* __restrict__ y_perm, const uint4* __restrict__ y_sh,
                    const float* __restrict__ w, const int32_t* __restrict__ perm_dst, int V,
                    int k, uint4* __restrict__ out, uint32_t* status, long long nk) {
+  pdl_wait();
+  pdl_launch();
   const int t = blockIdx.x;
   const long long tk = static_cast<long long>(t) * k, tv = static_cast<long long>(t) * V;
   combine_token(y_perm, y_sh ? y_sh + tv : nullptr, w + tk, perm_dst + tk, V, k, out + tv, status, nk);
@@ -329,6 +337,8 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtas)
     combine_mbox_kernel(const MboxRound* __restrict__ r, const MboxGeom g, const uint4* __restrict__ y_perm,
                         const uint4* __restrict__ y_sh, const float* __restrict__ w,
                         const int32_t* __restrict__ perm_dst, uint32_t* status) {
+  pdl_wait();
+  pdl_launch();
   const int n_total = r->n_total;
   const int V = g.H / 8;
   const long long nk = static_cast<long long>(n_total) * g.k;
@@ -387,10 +397,7 @@ cudaError_t launch_dispatch_seg(const void* x, int n, int H, int k, int E, const
                                 const int32_t* chunk_base, void* x_perm, int32_t* perm_src, int32_t* perm_dst,
                                 uint32_t* status, const DispatchSeg& seg, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  dispatch_kernel<false><<<n, kDispatchThreads, 0, s>>>(static_cast<const uint4*>(x), H / 8, k, E, idx, chunk_base,
-                                                        x_perm, nullptr, nullptr, nullptr, perm_src, perm_dst, status,
-                                                        seg);
-  return cudaGetLastError();
+  return launch_pdl(dispatch_kernel<false>, n, kDispatchThreads, 0, s, 1, static_cast<const uint4*>(x), H / 8, k, E, idx, chunk_base, x_perm, nullptr, nullptr, nullptr, perm_src, perm_dst, status, seg);
 }
 
 cudaError_t launch_dispatch_fp8(const void* x, int n, int H, int k, int E, const int32_t* idx,
@@ -410,52 +417,38 @@ cudaError_t launch_dispatch_fp8_seg(const void* x, int n, int H, int k, int E, c
                                     int32_t* perm_src, int32_t* perm_dst, uint32_t* status, const DispatchSeg& seg,
                                     cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  dispatch_kernel<true><<<n, kDispatchThreads, 0, s>>>(static_cast<const uint4*>(x), H / 8, k, E, idx, chunk_base, xq,
-                                                       xs, static_cast<uint2*>(xq_sh), xs_sh, perm_src, perm_dst,
-                                                       status, seg);
-  return cudaGetLastError();
+  return launch_pdl(dispatch_kernel<true>, n, kDispatchThreads, 0, s, 1, static_cast<const uint4*>(x), H / 8, k, E, idx, chunk_base, xq, xs, static_cast<uint2*>(xq_sh), xs_sh, perm_src, perm_dst, status, seg);
 }
 
 cudaError_t launch_quantize_rows(const void* x, int rows, int cols, void* q, float* s, cudaStream_t st) {
   if (rows <= 0) return cudaSuccess;
-  quantize_rows_kernel<<<ceil_div(rows, 8), 256, 0, st>>>(static_cast<const uint4*>(x), rows, cols / 8,
-                                                          static_cast<uint2*>(q), s);
-  return cudaGetLastError();
+  return launch_pdl(quantize_rows_kernel, ceil_div(rows, 8), 256, 0, st, 1, static_cast<const uint4*>(x), rows, cols / 8, static_cast<uint2*>(q), s);
 }
 
 cudaError_t launch_combine(const void* y_perm, const void* y_shared, const float* w,
                            const int32_t* perm_dst, int n, int H, int k, void* out, uint32_t* status,
                            cudaStream_t s, long long rows_total) {
   if (n <= 0) return cudaSuccess;
-  combine_kernel<<<n, kCombineThreads, 0, s>>>(
-      static_cast<const uint4*>(y_perm), static_cast<const uint4*>(y_shared), w, perm_dst, H / 8, k,
-      static_cast<uint4*>(out), status, rows_total > 0 ? rows_total : static_cast<long long>(n) * k);
-  return cudaGetLastError();
+  return launch_pdl(combine_kernel, n, kCombineThreads, 0, s, 1, static_cast<const uint4*>(y_perm), static_cast<const uint4*>(y_shared), w, perm_dst, H / 8, k, static_cast<uint4*>(out), status, rows_total > 0 ? rows_total : static_cast<long long>(n) * k);
 }
 
 cudaError_t launch_dispatch_mbox(const MboxRound* r, MboxGeom g, const int32_t* idx, const int32_t* chunk_base,
                                  const int32_t* offsets, void* x_perm, int32_t* perm_src, int32_t* perm_dst,
                                  void* x_sh, uint32_t* status, cudaStream_t s) {
   // one post's tokens; more loop
-  dispatch_mbox_kernel<false><<<g.slot_tokens, kDispatchThreads, 0, s>>>(r, g, idx, chunk_base, offsets, x_perm, nullptr,
-                                                                         x_sh, nullptr, perm_src, perm_dst, status);
-  return cudaGetLastError();
+  return launch_pdl(dispatch_mbox_kernel<false>, g.slot_tokens, kDispatchThreads, 0, s, 1, r, g, idx, chunk_base, offsets, x_perm, nullptr, x_sh, nullptr, perm_src, perm_dst, status);
 }
 
 cudaError_t launch_dispatch_fp8_mbox(const MboxRound* r, MboxGeom g, const int32_t* idx, const int32_t* chunk_base,
                                      const int32_t* offsets, void* xq, float* xs, void* xq_sh, float* xs_sh,
                                      int32_t* perm_src, int32_t* perm_dst, uint32_t* status, cudaStream_t s) {
-  dispatch_mbox_kernel<true><<<g.slot_tokens, kDispatchThreads, 0, s>>>(r, g, idx, chunk_base, offsets, xq, xs, xq_sh,
-                                                                        xs_sh, perm_src, perm_dst, status);
-  return cudaGetLastError();
+  return launch_pdl(dispatch_mbox_kernel<true>, g.slot_tokens, kDispatchThreads, 0, s, 1, r, g, idx, chunk_base, offsets, xq, xs, xq_sh, xs_sh, perm_src, perm_dst, status);
 }
 
 cudaError_t launch_combine_mbox(const MboxRound* r, MboxGeom g, const void* y_perm, const void* y_shared,
                                 const float* w, const int32_t* perm_dst, uint32_t* status, cudaStream_t s) {
   // one post's tokens; more loop
-  combine_mbox_kernel<<<g.slot_tokens, kCombineThreads, 0, s>>>(r, g, static_cast<const uint4*>(y_perm),
-                                                          static_cast<const uint4*>(y_shared), w, perm_dst, status);
-  return cudaGetLastError();
+  return launch_pdl(combine_mbox_kernel, g.slot_tokens, kCombineThreads, 0, s, 1, r, g, static_cast<const uint4*>(y_perm), static_cast<const uint4*>(y_shared), w, perm_dst, status);
 }
 
 cudaError_t launch_retile(const void* a, const void* b, int E, int R, long long row_bytes, bool gate_up, int log_unit,

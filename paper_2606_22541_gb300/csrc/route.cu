@@ -32,6 +32,8 @@ constexpr int kRouterAhead = 8;  // row pieces in flight per lane
 __global__ void __launch_bounds__(256) router_small_kernel(const uint4* __restrict__ x, LayerRef lref,
                                                            uint32_t* status, int n, int V, int E,
                                                            float* __restrict__ logits) {
+  pdl_wait();
+  pdl_launch();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x * 8 + warp;
   if (t >= n) return;
@@ -113,6 +115,8 @@ template <int NB>  // E = 8 NB experts
 __global__ void __launch_bounds__(kRmmaWarps * 32) router_mma_kernel(const uint4* __restrict__ x, LayerRef lref,
                                                                      uint32_t* status, int n, int V,
                                                                      float* __restrict__ logits) {
+  pdl_wait();
+  pdl_launch();
   constexpr int E = 8 * NB;
   __shared__ float part[kRmmaWarps][kRmmaTokens][E];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -187,6 +191,8 @@ __global__ void __launch_bounds__(kGateWarps * 32) gate_kernel(const float* __re
                                                                float* __restrict__ wout,
                                                                int32_t* __restrict__ hist, int n_chunks,
                                                                int chunk0) {
+  pdl_wait();
+  pdl_launch();
   __shared__ int shist[kMaxExperts];
   __shared__ float ssel[kGateWarps][kMaxExperts];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -390,6 +396,8 @@ __global__ void __launch_bounds__(kChunkTokens * T) gate_team_kernel(const float
                                                                  float* __restrict__ wout,
                                                                  int32_t* __restrict__ hist, int n_chunks,
                                                                  int chunk0) {
+  pdl_wait();
+  pdl_launch();
   static_assert(T * S <= kMaxExperts && (T == 8 || T == 16 || T == 32) && S <= 8, "team shape");
   __shared__ int shist[kMaxExperts];
   const int lane = threadIdx.x & 31;
@@ -559,6 +567,8 @@ __global__ void __launch_bounds__(kChunkTokens * T) gate_team_kernel(const float
 __global__ void __launch_bounds__(256) hist_kernel(const int32_t* __restrict__ idx, int n, int k, int E,
                                                    int32_t* __restrict__ hist, int n_chunks, uint32_t* status,
                                                    int32_t* ticket) {
+  pdl_wait();
+  pdl_launch();
   __shared__ int shist[kMaxExperts];
   if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;  // for the scan that follows
   for (int e = threadIdx.x; e < E; e += blockDim.x) shist[e] = 0;
@@ -627,6 +637,8 @@ __global__ void __launch_bounds__(kScanThreads) scan_kernel(const int32_t* __res
                                                             int32_t* __restrict__ ticket,
                                                             const int32_t* __restrict__ rowmap,
                                                             const int32_t* __restrict__ n_chunks_dev) {
+  pdl_wait();
+  pdl_launch();
   __shared__ int part[kScanWarps][32];
   __shared__ int swarp[33];
   __shared__ bool last;
@@ -687,6 +699,8 @@ __global__ void __launch_bounds__(kScanThreads) scan_kernel(const int32_t* __res
 // Sum of the K-slice planes of the router GEMM, added in slice order.
 __global__ void reduce_splits_kernel(const float* __restrict__ parts, int splits, long long plane,
                                      float* __restrict__ out) {
+  pdl_wait();
+  pdl_launch();
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < plane;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
     float v = parts[i];
@@ -705,8 +719,8 @@ cudaError_t launch_router_small(const void* x, const LayerRef& lref, int n, int 
     const uint4* xv = static_cast<const uint4*>(x);
 #define ASAP_ROUTER_MMA(NBV)                                                                                  \
   if (E == 8 * NBV) {                                                                                         \
-    router_mma_kernel<NBV><<<grid, kRmmaWarps * 32, 0, s>>>(xv, lref, status, n, H / 8, logits);              \
-    return cudaGetLastError();                                                                                \
+    return launch_pdl(router_mma_kernel<NBV>, grid, kRmmaWarps * 32, 0, s, 1, xv, lref, status, n, H / 8,     \
+                      logits);                                                                                \
   }
     ASAP_ROUTER_MMA(1)
     ASAP_ROUTER_MMA(2)
@@ -714,9 +728,7 @@ cudaError_t launch_router_small(const void* x, const LayerRef& lref, int n, int 
     ASAP_ROUTER_MMA(8)
 #undef ASAP_ROUTER_MMA
   }
-  router_small_kernel<<<ceil_div(n, 8), 256, 0, s>>>(static_cast<const uint4*>(x), lref, status, n, H / 8, E,
-                                                       logits);
-  return cudaGetLastError();
+  return launch_pdl(router_small_kernel, ceil_div(n, 8), 256, 0, s, 1, static_cast<const uint4*>(x), lref, status, n, H / 8, E, logits);
 }
 
 cudaError_t launch_gate(const float* logits, int splits, int n, const GateParams& p, int32_t* idx, float* w,
@@ -740,9 +752,8 @@ cudaError_t launch_gate_seg(const float* logits, int splits, int n, const GatePa
   if (team) {
 #define ASAP_GATE_TEAM(TV, SV)                                                                                  \
   if (T == TV && S == SV) {                                                                                     \
-    gate_team_kernel<TV, SV><<<chunks, kChunkTokens * TV, 0, s>>>(logits, splits, plane, n, p, idx, w, hist,    \
-                                                                  n_chunks_total, chunk0);                      \
-    return cudaGetLastError();                                                                                  \
+    return launch_pdl(gate_team_kernel<TV, SV>, chunks, kChunkTokens * TV, 0, s, 1, logits, splits, plane, n,   \
+                      p, idx, w, hist, n_chunks_total, chunk0);                                                 \
   }
     ASAP_GATE_TEAM(32, 8)
     ASAP_GATE_TEAM(32, 4)
@@ -752,38 +763,31 @@ cudaError_t launch_gate_seg(const float* logits, int splits, int n, const GatePa
     ASAP_GATE_TEAM(8, 1)
 #undef ASAP_GATE_TEAM
   }
-  gate_kernel<<<chunks, kGateWarps * 32, 0, s>>>(logits, splits, plane, n, p, idx, w, hist, n_chunks_total, chunk0);
-  return cudaGetLastError();
+  return launch_pdl(gate_kernel, chunks, kGateWarps * 32, 0, s, 1, logits, splits, plane, n, p, idx, w, hist, n_chunks_total, chunk0);
 }
 
 cudaError_t launch_hist(const int32_t* idx, int n, int k, int E, int32_t* hist, uint32_t* status, int32_t* ticket,
                         cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const int chunks = ceil_div(n, kChunkTokens);
-  hist_kernel<<<chunks, 256, 0, s>>>(idx, n, k, E, hist, chunks, status, ticket);
-  return cudaGetLastError();
+  return launch_pdl(hist_kernel, chunks, 256, 0, s, 1, idx, n, k, E, hist, chunks, status, ticket);
 }
 
 cudaError_t launch_reduce_splits(const float* parts, int splits, long long plane, float* out, cudaStream_t s) {
   if (plane <= 0) return cudaSuccess;
   const int blocks = static_cast<int>(std::min<long long>((plane + 255) / 256, 4096));
-  reduce_splits_kernel<<<blocks, 256, 0, s>>>(parts, splits, plane, out);
-  return cudaGetLastError();
+  return launch_pdl(reduce_splits_kernel, blocks, 256, 0, s, 1, parts, splits, plane, out);
 }
 
 cudaError_t launch_scan(const int32_t* hist, int n_chunks, int E, int32_t* counts, int32_t* offsets,
                         int32_t* chunk_base, int32_t* ticket, cudaStream_t s, int32_t* tile_counters) {
-  scan_kernel<false><<<ceil_div(E, 32), kScanThreads, 0, s>>>(hist, n_chunks, E, counts, offsets, chunk_base,
-                                                             tile_counters, ticket, nullptr, nullptr);
-  return cudaGetLastError();
+  return launch_pdl(scan_kernel<false>, ceil_div(E, 32), kScanThreads, 0, s, 1, hist, n_chunks, E, counts, offsets, chunk_base, tile_counters, ticket, nullptr, nullptr);
 }
 
 cudaError_t launch_scan_mapped(const int32_t* hist, const int32_t* rowmap, const int32_t* n_chunks, int max_chunks,
                                int E, int32_t* counts, int32_t* offsets, int32_t* chunk_base, int32_t* ticket,
                                int32_t* tile_counters, cudaStream_t s) {
-  scan_kernel<true><<<ceil_div(E, 32), kScanThreads, 0, s>>>(hist, max_chunks, E, counts, offsets, chunk_base,
-                                                            tile_counters, ticket, rowmap, n_chunks);
-  return cudaGetLastError();
+  return launch_pdl(scan_kernel<true>, ceil_div(E, 32), kScanThreads, 0, s, 1, hist, max_chunks, E, counts, offsets, chunk_base, tile_counters, ticket, rowmap, n_chunks);
 }
 
 }  // namespace asap

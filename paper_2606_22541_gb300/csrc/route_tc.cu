@@ -157,12 +157,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   const CUtensorMap* tmW = nullptr;
 
   if (warp == 0) {
-    const LayerEntry& le =
-        a.lref.table[load_layer(a.lref.layer, a.lref.n_layers, a.status, blockIdx.x == 0 && lane == 0)];
-    tmW = &le.map[MAP_ROUTER];
-    tensormap_acquire(tmW);
     if (lane == 0) {
-      *bias_slot = le.router_bias;
       for (int s = 0; s < kRA; ++s) {
         mbar_init(fullA(s), 1);
         mbar_init(emptyA(s), 1);
@@ -179,6 +174,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       *acc_bad = aligned ? 0 : 1;
       fence_barrier_init();
       tma_prefetch_desc(&tmX);
+    }
+    pdl_wait();
+    pdl_launch();
+    const LayerEntry& le =
+        a.lref.table[load_layer(a.lref.layer, a.lref.n_layers, a.status, blockIdx.x == 0 && lane == 0)];
+    tmW = &le.map[MAP_ROUTER];
+    tensormap_acquire(tmW);
+    if (lane == 0) {
+      *bias_slot = le.router_bias;
       tma_prefetch_desc(tmW);
       if (!aligned) record_status(a.status, ST_SMEM_ALIGN);
     }
@@ -186,6 +190,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tmem_alloc(smem_u32(tmem_slot), tmem_cols);
     tmem_relinquish();
   }
+  pdl_wait();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -618,19 +623,7 @@ cudaError_t launch_route_fused(const CUtensorMap& tmX, const RouteFusedArgs& a, 
       a.top_k < 1 || a.top_k > kMaxTopK || a.k_iters < a.splits ||
       !(a.seq_slices <= 1 || (a.splits == 1 && (a.seq_slices == 2 || a.seq_slices == 4) && a.k_iters >= a.seq_slices)))
     return cudaErrorInvalidValue;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(ceil_div(a.n, kGemmBM) * a.splits);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = kSmem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = static_cast<unsigned>(a.splits);
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, route_fused_kernel, tmX, a);
+  return launch_pdl(route_fused_kernel, dim3(ceil_div(a.n, kGemmBM) * a.splits), dim3(kThreads), kSmem, s, a.splits, tmX, a);
 }
 
 }  // namespace asap
