@@ -73,7 +73,7 @@ constexpr int kHintA = ASAP_HINT_BF16_A, kHintB = ASAP_HINT_BF16_B, kHintDnA = A
 constexpr int kHintF8A = ASAP_HINT_FP8_A, kHintF8B = ASAP_HINT_FP8_B;
 
 struct Layout {
-  size_t logits, idx, w, hist, chunk_base, counts, offsets, perm_src, perm_dst, tile_counters, ticket;
+  size_t logits, idx, w, hist, chunk_base, counts, offsets, perm_src, perm_dst, tile_counters;
   // bf16: x_perm (also y_perm in asap_moe_layer), h, h_sh, y_sh
   size_t x_perm, h, h_sh, y_sh, comb_cnt;
   // fp8: quantised rows and their per-128-channel scales, bf16 expert outputs
@@ -104,7 +104,6 @@ Layout layout(const asap_moe_config& c, long long n) {
   L.perm_src = take(nk * 4);
   L.perm_dst = take(nk * 4);
   L.tile_counters = take(asap::kTileCounters * 4);
-  L.ticket = take(4);
   if (c.dtype == ASAP_FP8_E4M3_BLOCK128) {
     L.xq = take(nk * H);
     L.xs = take(nk * (H / 128) * 4);
@@ -174,25 +173,21 @@ int router_splits(asap_moe_t h, int n) {
   return p;
 }
 
-// Routing in one launch (router GEMM + gating + scan): E = 256 with grouped
-// sigmoid gating in 1, 2, 4 or 8 groups.  Other configurations run the
-// router, gate and scan kernels one after the other.
+// Router GEMM, gating and histogram in one launch: E = 256 with grouped sigmoid
+// gating in 1, 2, 4 or 8 groups.  Other configurations run the router and gate
+// kernels one after the other.  The scan follows in both.
 bool fused_route(asap_moe_t h) {
   const asap_moe_config& c = h->cfg;
   return h->tc_router && c.gating == ASAP_GATE_SIGMOID_GROUPED &&
          (c.n_groups == 1 || c.n_groups == 2 || c.n_groups == 4 || c.n_groups == 8);
 }
 
-// The fused route launch for n tokens of x.  With ticket (zero at launch)
-// its last CTA scans the histogram into chunk_base, counts and offsets and
-// zeroes tile_counters (nullable); without, hist columns [chunk0, chunk0 +
-// ceil(n/32)) of n_chunks_total are left for one scan over several
-// micro-batches.
+// The fused route launch for n tokens of x: idx, w and the histogram rows
+// [chunk0, chunk0 + ceil(n/32)); a scan follows.
 // narrow: no cluster; each CTA computes its tile's K slices one after the
 // other (same logits bits), so concurrent routes share the GPU in one wave.
 int run_route_fused(asap_moe_t h, const void* x, int n, int32_t* idx, float* w, int32_t* hist, int chunk0,
-                    int n_chunks_total, int32_t* ticket, int32_t* counts, int32_t* offsets, int32_t* chunk_base,
-                    int32_t* tile_counters, const int32_t* layer, cudaStream_t st, bool narrow = false);
+                    const int32_t* layer, cudaStream_t st, bool narrow = false);
 
 // Router logits as ``splits`` planes of partial sums [splits][n][E] (planes
 // are added in order by the consumer); splits == 1 writes the logits.
@@ -232,8 +227,7 @@ int run_router_logits(asap_moe_t h, const void* x, int n, float* logits, int spl
 }
 
 int run_route_fused(asap_moe_t h, const void* x, int n, int32_t* idx, float* w, int32_t* hist, int chunk0,
-                    int n_chunks_total, int32_t* ticket, int32_t* counts, int32_t* offsets, int32_t* chunk_base,
-                    int32_t* tile_counters, const int32_t* layer, cudaStream_t st, bool narrow) {
+                    const int32_t* layer, cudaStream_t st, bool narrow) {
   const asap_moe_config& c = h->cfg;
   CUtensorMap tmx;
   std::string err;
@@ -254,12 +248,6 @@ int run_route_fused(asap_moe_t h, const void* x, int n, int32_t* idx, float* w, 
   a.w = w;
   a.hist = hist;
   a.chunk0 = chunk0;
-  a.n_chunks_total = n_chunks_total;
-  a.ticket = ticket;
-  a.counts = counts;
-  a.offsets = offsets;
-  a.chunk_base = chunk_base;
-  a.tile_counters = tile_counters;
   CU_TRY(asap::launch_route_fused(tmx, a, st), "fused route launch");
   return ASAP_OK;
 }
@@ -270,8 +258,7 @@ int run_route_fused(asap_moe_t h, const void* x, int n, int32_t* idx, float* w, 
 int run_route(asap_moe_t h, const void* x, int n, int32_t* idx, float* w, int32_t* counts, int32_t* offsets,
               void* ws, const int32_t* layer, cudaStream_t st);
 
-// ticket: the scan's ticket in the call's scratch (zeroed by the gate launch).
-asap::GateParams gate_params(asap_moe_t h, const int32_t* layer, int32_t* ticket) {
+asap::GateParams gate_params(asap_moe_t h, const int32_t* layer) {
   const asap_moe_config& c = h->cfg;
   asap::GateParams p{};
   p.n_experts = c.n_experts;
@@ -282,7 +269,6 @@ asap::GateParams gate_params(asap_moe_t h, const int32_t* layer, int32_t* ticket
   p.route_scale = c.route_scale;
   p.lref = lref(h, layer);
   p.status = h->status;
-  p.ticket = ticket;
   return p;
 }
 
@@ -291,10 +277,9 @@ int run_gate_scan(asap_moe_t h, const float* logits, int splits, int n, int32_t*
   const Layout L = layout(h->cfg, n);
   int32_t* hist = at<int32_t>(ws, L.hist);
   int32_t* base = at<int32_t>(ws, L.chunk_base);
-  int32_t* ticket = at<int32_t>(ws, L.ticket);
-  CU_TRY(asap::launch_gate(logits, splits, n, gate_params(h, layer, ticket), idx, w, hist, st), "gate launch");
-  CU_TRY(asap::launch_scan(hist, asap::ceil_div(n, asap::kChunkTokens), h->cfg.n_experts, counts, offsets, base,
-                           ticket, st, at<int32_t>(ws, L.tile_counters)),
+  CU_TRY(asap::launch_gate(logits, splits, n, gate_params(h, layer), idx, w, hist, st), "gate launch");
+  CU_TRY(asap::launch_scan(hist, asap::ceil_div(n, asap::kChunkTokens), h->cfg.n_experts, counts, offsets, base, st,
+                           at<int32_t>(ws, L.tile_counters)),
          "scan launch");
   return ASAP_OK;
 }
@@ -303,12 +288,12 @@ int run_route(asap_moe_t h, const void* x, int n, int32_t* idx, float* w, int32_
               void* ws, const int32_t* layer, cudaStream_t st) {
   const Layout L = layout(h->cfg, n);
   if (fused_route(h)) {
-    // the tile counters and the ticket, one memset (the ticket follows them)
-    static_assert(asap::kTileCounters * 4 <= 256, "tile counters fit before the ticket");
-    CU_TRY(cudaMemsetAsync(at<char>(ws, L.tile_counters), 0, L.ticket - L.tile_counters + 4, st), "ticket");
-    return run_route_fused(h, x, n, idx, w, at<int32_t>(ws, L.hist), 0, asap::ceil_div(n, asap::kChunkTokens),
-                           at<int32_t>(ws, L.ticket), counts, offsets, at<int32_t>(ws, L.chunk_base),
-                           at<int32_t>(ws, L.tile_counters), layer, st);
+    int r = run_route_fused(h, x, n, idx, w, at<int32_t>(ws, L.hist), 0, layer, st);
+    if (r != ASAP_OK) return r;
+    CU_TRY(asap::launch_scan(at<int32_t>(ws, L.hist), asap::ceil_div(n, asap::kChunkTokens), h->cfg.n_experts, counts,
+                             offsets, at<int32_t>(ws, L.chunk_base), st, at<int32_t>(ws, L.tile_counters)),
+           "scan launch");
+    return ASAP_OK;
   }
   float* logits = at<float>(ws, L.logits);
   const int splits = router_splits(h, n);
@@ -959,10 +944,9 @@ ASAP_API int asap_moe_dispatch(asap_moe_t h, const void* x, int32_t n, const int
   cudaStream_t st = S(stream);
   int32_t* hist = at<int32_t>(ws, L.hist);
   int32_t* base = at<int32_t>(ws, L.chunk_base);
-  int32_t* ticket = at<int32_t>(ws, L.ticket);
   int32_t* offs = at<int32_t>(ws, L.offsets);
-  CU_TRY(asap::launch_hist(idx, n, c.top_k, c.n_experts, hist, h->status, ticket, st), "hist launch");
-  CU_TRY(asap::launch_scan(hist, chunks, c.n_experts, at<int32_t>(ws, L.counts), offs, base, ticket, st),
+  CU_TRY(asap::launch_hist(idx, n, c.top_k, c.n_experts, hist, h->status, st), "hist launch");
+  CU_TRY(asap::launch_scan(hist, chunks, c.n_experts, at<int32_t>(ws, L.counts), offs, base, st),
          "scan launch");
   if (h->fp8)
     CU_TRY(asap::launch_dispatch_fp8(x, n, c.hidden, c.top_k, c.n_experts, idx, base, offs, x_perm, x_perm_scales,
@@ -1202,14 +1186,13 @@ int run_layer_batched(asap_moe_t h, int32_t count, const void* const* xs, const 
     const int n = ns[i];
     if (n > 0 && fused_route(h)) {
       if ((r = run_route_fused(h, xs[i], n, idx + static_cast<long long>(tok0) * k,
-                               w + static_cast<long long>(tok0) * k, hist, chunk0, chunks_total, nullptr, nullptr,
-                               nullptr, nullptr, nullptr, layer, st)) != ASAP_OK)
+                               w + static_cast<long long>(tok0) * k, hist, chunk0, layer, st)) != ASAP_OK)
         return r;
     } else if (n > 0) {
       const int splits = router_splits(h, n);
       float* lg = logits + static_cast<long long>(asap::kMaxRouterSplits) * tok0 * E;
       if ((r = run_router_logits(h, xs[i], n, lg, splits, layer, st)) != ASAP_OK) return r;
-      CU_TRY(asap::launch_gate_seg(lg, splits, n, gate_params(h, layer, at<int32_t>(ws, L.ticket)),
+      CU_TRY(asap::launch_gate_seg(lg, splits, n, gate_params(h, layer),
                                    idx + static_cast<long long>(tok0) * k,
                                    w + static_cast<long long>(tok0) * k, hist, chunk0, chunks_total, st),
              "gate launch");
@@ -1218,11 +1201,9 @@ int run_layer_batched(asap_moe_t h, int32_t count, const void* const* xs, const 
     chunk0 += asap::ceil_div(n, asap::kChunkTokens);
   }
   // one histogram scan over every chunk: expert segments hold the rows of all
-  // micro-batches, in (micro-batch, token, slot) order (the scan's ticket is
-  // zero at launch: the gate kernels zero it, the fused route does not)
-  if (fused_route(h)) CU_TRY(cudaMemsetAsync(at<int32_t>(ws, L.ticket), 0, 4, st), "ticket");
-  CU_TRY(asap::launch_scan(hist, chunks_total, E, at<int32_t>(ws, L.counts), offsets, base, at<int32_t>(ws, L.ticket),
-                           st, at<int32_t>(ws, L.tile_counters)),
+  // micro-batches, in (micro-batch, token, slot) order
+  CU_TRY(asap::launch_scan(hist, chunks_total, E, at<int32_t>(ws, L.counts), offsets, base, st,
+                           at<int32_t>(ws, L.tile_counters)),
          "scan launch");
   void* y_sh = c.n_shared ? at<void>(ws, L.y_sh) : nullptr;
   tok0 = 0;
@@ -1541,15 +1522,15 @@ ASAP_API int asap_moe_mailbox_post(asap_moe_mailbox_t m, int32_t slot, const voi
     // routing exactly as asap_moe_route routes n tokens; the histogram rows
     // are the slot's, scanned later together with the other claimed posts
     if (fused_route(h)) {
-      if ((r = run_route_fused(h, x, n, idx, w, hist, chunk0, chunks_total, nullptr, nullptr, nullptr, nullptr,
-                               nullptr, layer, st, /*narrow=*/true)) != ASAP_OK)
+      if ((r = run_route_fused(h, x, n, idx, w, hist, chunk0, layer, st,
+                               /*narrow=*/true)) != ASAP_OK)
         return r;
     } else {
       const int splits = router_splits(h, n);
       float* lg = at<float>(m->ws, m->L.logits) +
                   static_cast<long long>(slot) * asap::kMaxRouterSplits * g.slot_tokens * c.n_experts;
       if ((r = run_router_logits(h, x, n, lg, splits, layer, st)) != ASAP_OK) return r;
-      CU_TRY(asap::launch_gate_seg(lg, splits, n, gate_params(h, layer, nullptr), idx, w, hist, chunk0,
+      CU_TRY(asap::launch_gate_seg(lg, splits, n, gate_params(h, layer), idx, w, hist, chunk0,
                                    chunks_total, st),
              "gate launch");
     }
@@ -1590,12 +1571,11 @@ int serve_round(asap_moe_mailbox_t m, int count, const int32_t* slots, const uin
   // server workspace
   for (int i = 0; i < count; ++i) CU_TRY(cudaStreamWaitEvent(st, m->post_ev[slots[i]], 0), "wait for the post");
   if (m->any_round) CU_TRY(cudaStreamWaitEvent(st, m->round_ev, 0), "wait for the previous round");
-  CU_TRY(asap::launch_mbox_claim(m->slots, g, slot, epoch, m->wait_ns, m->round, m->rowmap, at<int32_t>(ws, L.ticket),
-                                 h->status, st),
+  CU_TRY(asap::launch_mbox_claim(m->slots, g, slot, epoch, m->wait_ns, m->round, m->rowmap, h->status, st),
          "claim launch");
   CU_TRY(asap::launch_scan_mapped(at<int32_t>(ws, L.hist), m->rowmap, &m->round->chunks_total,
                                   g.n_slots * g.slot_chunks, c.n_experts, at<int32_t>(ws, L.counts), offsets,
-                                  at<int32_t>(ws, L.chunk_base), at<int32_t>(ws, L.ticket), counters, st),
+                                  at<int32_t>(ws, L.chunk_base), counters, st),
          "scan launch");
   const int32_t* idx = at<int32_t>(ws, L.idx);
   int32_t* perm_dst = at<int32_t>(ws, L.perm_dst);
@@ -1750,7 +1730,7 @@ constexpr size_t kStaticLogitsBytes = static_cast<size_t>(asap::kMaxRouterSplits
                                       ASAP_MOE_MAX_EXPERTS * sizeof(float);  // 16 MiB
 constexpr size_t kStaticChunkBytes = static_cast<size_t>(kStaticRouteMaxTokens / asap::kChunkTokens) *
                                      ASAP_MOE_MAX_EXPERTS * sizeof(int32_t);                  // 128 KiB
-constexpr size_t kStaticRouteBytes = kStaticLogitsBytes + 2 * kStaticChunkBytes + 256;  // + the scan's ticket
+constexpr size_t kStaticRouteBytes = kStaticLogitsBytes + 2 * kStaticChunkBytes;
 
 constexpr int kStaticMaxDevices = 64;
 std::mutex g_static_route_mu;
@@ -1802,25 +1782,23 @@ ASAP_API int asap_moe_route_noalloc(asap_moe_t h, const void* x, int32_t n, int3
   int32_t* hist = reinterpret_cast<int32_t*>(scratch + kStaticLogitsBytes);
   int32_t* base = reinterpret_cast<int32_t*>(scratch + kStaticLogitsBytes + kStaticChunkBytes);
   cudaStream_t st = S(stream);
-  int32_t* ticket = reinterpret_cast<int32_t*>(scratch + kStaticLogitsBytes + 2 * kStaticChunkBytes);
+  auto scan = [&]() -> int {
+    CU_TRY(asap::launch_scan(hist, asap::ceil_div(n, asap::kChunkTokens), h->cfg.n_experts, counts, offsets, base, st),
+           "scan launch");
+    return ASAP_OK;
+  };
   if (fused_route(h)) {
-    // the same single launch as asap_moe_route (same K slices, same bits);
-    // its ticket must start at zero, the rest is written before it is read
-    CU_TRY(cudaMemsetAsync(ticket, 0, sizeof(int32_t), st), "ticket");
-    return run_route_fused(h, x, n, idx, w, hist, 0, asap::ceil_div(n, asap::kChunkTokens), ticket, counts, offsets,
-                           base, nullptr, h->layer_ids, st);
+    // the same launches as asap_moe_route (same K slices, same bits)
+    if ((r = run_route_fused(h, x, n, idx, w, hist, 0, h->layer_ids, st)) != ASAP_OK) return r;
+    return scan();
   }
   // the router's K slices and their order of addition are those of
   // asap_moe_route, so the bits are the same.  Every scratch element read
   // below is written earlier on the same stream (the logit planes by the
-  // router, all E entries of each chunk's histogram and the scan's ticket by
-  // the gate kernel), so nothing has to be cleared between calls.
+  // router, all E entries of each chunk's histogram by the gate kernel), so
+  // nothing has to be cleared between calls.
   const int splits = router_splits(h, n);
   if ((r = run_router_logits(h, x, n, logits, splits, h->layer_ids, st)) != ASAP_OK) return r;
-  CU_TRY(asap::launch_gate(logits, splits, n, gate_params(h, h->layer_ids, ticket), idx, w, hist, st),
-         "gate launch");
-  CU_TRY(asap::launch_scan(hist, asap::ceil_div(n, asap::kChunkTokens), h->cfg.n_experts, counts, offsets, base,
-                           ticket, st),
-         "scan launch");
-  return ASAP_OK;
+  CU_TRY(asap::launch_gate(logits, splits, n, gate_params(h, h->layer_ids), idx, w, hist, st), "gate launch");
+  return scan();
 }

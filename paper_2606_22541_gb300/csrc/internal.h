@@ -170,7 +170,6 @@ struct GateParams {
   float route_scale;
   LayerRef lref;  // selection bias: table[layer].router_bias ([E] or nullptr)
   uint32_t* status;
-  int32_t* ticket;  // the scan's ticket, zeroed by the gate launch (nullable)
 };
 // Router on the CUDA cores (E < 256): weights table[layer].router_w.
 cudaError_t launch_router_small(const void* x, const LayerRef& lref, int n, int H, int E, float* logits,
@@ -185,25 +184,22 @@ cudaError_t launch_reduce_splits(const float* parts, int splits, long long plane
 // n_chunks_total rows.
 cudaError_t launch_gate_seg(const float* logits, int splits, int n, const GateParams& p, int32_t* idx, float* w,
                             int32_t* hist, int chunk0, int n_chunks_total, cudaStream_t s);
-// hist as launch_gate writes it; zeroes the scan's ticket.
-cudaError_t launch_hist(const int32_t* idx, int n, int k, int E, int32_t* hist, uint32_t* status, int32_t* ticket,
+// hist as launch_gate writes it.
+cudaError_t launch_hist(const int32_t* idx, int n, int k, int E, int32_t* hist, uint32_t* status,
                         cudaStream_t s);
 // counts, offsets, and chunk_base[c][e] = entries of expert e in chunks
 // before c (relative: the absolute base is offsets[e] + chunk_base[c][e]);
 // hist and chunk_base are chunk-major [n_chunks][E].
-// ticket: one int, zero at launch (the gate / hist launch zeroes it), left
-// zero.  tile_counters (nullable): kTileCounters ints zeroed for the grouped
-// GEMMs that follow on the stream.
+// tile_counters (nullable): kTileCounters ints zeroed for the grouped GEMMs that
+// follow on the stream.
 cudaError_t launch_scan(const int32_t* hist, int n_chunks, int E, int32_t* counts, int32_t* offsets,
-                        int32_t* chunk_base, int32_t* ticket, cudaStream_t s, int32_t* tile_counters = nullptr);
+                        int32_t* chunk_base, cudaStream_t s, int32_t* tile_counters = nullptr);
 
-// Routing of one micro-batch in one launch (E = 256 on the tensor core,
-// grouped sigmoid gating with 1, 2, 4 or 8 groups): router logits over
-// ``splits`` K slices (a cluster of that many CTAs per 128-token tile, slices
-// added in order), gating, idx / w, the chunk-major histogram of its chunks
-// (rows chunk0 + c of n_chunks_total) and, when ticket is non-null, the
-// scan into chunk_base, counts and offsets by the last CTA (ticket zero at
-// launch, left zero) which also zeroes tile_counters (nullable).
+// Routing of one micro-batch up to the histogram in one launch (E = 256 on the
+// tensor core, grouped sigmoid gating with 1, 2, 4 or 8 groups): router logits
+// over ``splits`` K slices (a cluster of that many CTAs per 128-token tile,
+// slices added in order), gating, idx / w and the chunk-major histogram of its
+// chunks (rows chunk0 + c); a scan follows.
 constexpr int kRouteExperts = 256;
 struct RouteFusedArgs {
   LayerRef lref;  // router weights: table[layer].map[MAP_ROUTER]; selection bias
@@ -218,12 +214,7 @@ struct RouteFusedArgs {
   int32_t* idx;
   float* w;
   int32_t* hist;
-  int chunk0, n_chunks_total;
-  int32_t* ticket;
-  int32_t* counts;
-  int32_t* offsets;
-  int32_t* chunk_base;
-  int32_t* tile_counters;
+  int chunk0;
 };
 cudaError_t route_fused_set_attributes();
 // tmX: x [n, H] for [128, 64] boxes (encode_tmap_bf16).
@@ -328,16 +319,15 @@ cudaError_t launch_mbox_publish(MboxSlot* slots, int slot, const void* x, int n,
 // published epoch own_epoch (own_slot < 0: no wait; a wait that runs out
 // records ST_MBOX_WAIT), then claim every slot with posted > served whose post
 // belongs to the same layer as that post (after a wait that ran out: as the
-// lowest pending slot's post) into *r, write the histogram row map, zero the
-// scan's ticket.
+// lowest pending slot's post) into *r and write the histogram row map.
 cudaError_t launch_mbox_claim(MboxSlot* slots, MboxGeom g, int own_slot, unsigned long long own_epoch,
-                              unsigned long long wait_ns, MboxRound* r, int32_t* rowmap, int32_t* ticket,
-                              uint32_t* status, cudaStream_t s);
+                              unsigned long long wait_ns, MboxRound* r, int32_t* rowmap, uint32_t* status,
+                              cudaStream_t s);
 // The scan over the histogram rows rowmap[0 .. *n_chunks) (chunk_base written
 // at the same rows), otherwise as launch_scan.
 cudaError_t launch_scan_mapped(const int32_t* hist, const int32_t* rowmap, const int32_t* n_chunks, int max_chunks,
-                               int E, int32_t* counts, int32_t* offsets, int32_t* chunk_base, int32_t* ticket,
-                               int32_t* tile_counters, cudaStream_t s);
+                               int E, int32_t* counts, int32_t* offsets, int32_t* chunk_base, int32_t* tile_counters,
+                               cudaStream_t s);
 // Dispatch of every claimed post into the combined expert segments (rows in
 // (claimed slot, token, slot of k) order); perm_src holds combined token
 // indices, perm_dst the slot's own region; x_sh / xq_sh, xs_sh receive the

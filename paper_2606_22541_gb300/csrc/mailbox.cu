@@ -62,8 +62,7 @@ __global__ void mbox_publish_kernel(MboxSlot* slots, int slot, const void* x, in
 __global__ void __launch_bounds__(kMboxMaxSlots) mbox_claim_kernel(MboxSlot* slots, const MboxGeom g, int own_slot,
                                                                    unsigned long long own_epoch,
                                                                    unsigned long long wait_ns, MboxRound* r,
-                                                                   int32_t* rowmap, int32_t* ticket,
-                                                                   uint32_t* status) {
+                                                                   int32_t* rowmap, uint32_t* status) {
   __shared__ int s_cnt[2], s_tok[2], s_chk[2];
   __shared__ int s_layer, s_first;
   const int s = threadIdx.x, lane = s & 31, warp = s >> 5;
@@ -144,7 +143,6 @@ __global__ void __launch_bounds__(kMboxMaxSlots) mbox_claim_kernel(MboxSlot* slo
     r->chunks_total = ih;
     r->layer = layer;
     r->rounds += 1;
-    *ticket = 0;  // the scan that follows counts its CTAs on it
   }
 }
 
@@ -175,9 +173,9 @@ cudaError_t launch_mbox_publish(MboxSlot* slots, int slot, const void* x, int n,
 }
 
 cudaError_t launch_mbox_claim(MboxSlot* slots, MboxGeom g, int own_slot, unsigned long long own_epoch,
-                              unsigned long long wait_ns, MboxRound* r, int32_t* rowmap, int32_t* ticket,
-                              uint32_t* status, cudaStream_t s) {
-  mbox_claim_kernel<<<1, kMboxMaxSlots, 0, s>>>(slots, g, own_slot, own_epoch, wait_ns, r, rowmap, ticket, status);
+                              unsigned long long wait_ns, MboxRound* r, int32_t* rowmap, uint32_t* status,
+                              cudaStream_t s) {
+  mbox_claim_kernel<<<1, kMboxMaxSlots, 0, s>>>(slots, g, own_slot, own_epoch, wait_ns, r, rowmap, status);
   return cudaGetLastError();
 }
 

@@ -200,7 +200,6 @@ __global__ void __launch_bounds__(kGateWarps * 32) gate_kernel(const float* __re
   for (int e = threadIdx.x; e < E; e += blockDim.x) shist[e] = 0;
   __syncthreads();
 
-  if (p.ticket && blockIdx.x == 0 && threadIdx.x == 0) *p.ticket = 0;  // for the scan that follows
   const int t0 = blockIdx.x * kChunkTokens;
   const int t1 = min(n, t0 + kChunkTokens);
   const bool grouped = p.gating == 2;
@@ -404,7 +403,6 @@ __global__ void __launch_bounds__(kChunkTokens * T) gate_team_kernel(const float
   const int q = lane & (T - 1);  // lane in team
   const int E = T * S, k = p.top_k;
   for (int e = threadIdx.x; e < E; e += blockDim.x) shist[e] = 0;
-  if (p.ticket && blockIdx.x == 0 && threadIdx.x == 0) *p.ticket = 0;  // for the scan that follows
   __syncthreads();
   const bool grouped = p.gating == 2;
   const float* __restrict__ bias =
@@ -565,12 +563,10 @@ __global__ void __launch_bounds__(kChunkTokens * T) gate_team_kernel(const float
 
 // ------------------------------------------------------------ histogram only
 __global__ void __launch_bounds__(256) hist_kernel(const int32_t* __restrict__ idx, int n, int k, int E,
-                                                   int32_t* __restrict__ hist, int n_chunks, uint32_t* status,
-                                                   int32_t* ticket) {
+                                                   int32_t* __restrict__ hist, uint32_t* status) {
   pdl_wait();
   pdl_launch();
   __shared__ int shist[kMaxExperts];
-  if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0;  // for the scan that follows
   for (int e = threadIdx.x; e < E; e += blockDim.x) shist[e] = 0;
   __syncthreads();
   const int t0 = blockIdx.x * kChunkTokens;
@@ -585,115 +581,99 @@ __global__ void __launch_bounds__(256) hist_kernel(const int32_t* __restrict__ i
 }
 
 // ------------------------------------------------------------ scan
-// hist and chunk_base are chunk-major ([n_chunks][E]).  CTA g handles experts
-// 32g .. 32g+31 (lane = expert) and its 8 warps consecutive ranges of chunks:
-// each warp sums its range (128-byte rows), the warps' sums are combined in
-// shared memory, then each warp writes chunk_base[c][e] = the entries of
-// expert e in chunks before c (relative to the expert's offset, which
-// dispatch adds) over its range.  The last CTA to finish (ticket counter,
-// zero at launch, reset here) scans the counts into the exclusive offsets and
-// clears the grouped GEMMs' tile counters.
-constexpr int kScanThreads = 256;
-constexpr int kScanWarps = kScanThreads / 32;
-
-__device__ __forceinline__ int block_exclusive_scan(int v, int* swarp, int& total) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int incl = v;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int u = __shfl_up_sync(kFull, incl, o);
-    if (lane >= o) incl += u;
-  }
-  if (lane == 31) swarp[warp] = incl;
-  __syncthreads();
-  if (warp == 0) {
-    const int nw = blockDim.x >> 5;
-    int w = lane < nw ? swarp[lane] : 0;
-    int wi = w;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int u = __shfl_up_sync(kFull, wi, o);
-      if (lane >= o) wi += u;
-    }
-    if (lane < nw) swarp[lane] = wi - w;
-    if (lane == nw - 1) swarp[32] = wi;
-  }
-  __syncthreads();
-  total = swarp[32];
-  const int r = swarp[warp] + incl - v;
-  __syncthreads();  // swarp may be reused by the caller
-  return r;
-}
+// hist and chunk_base are chunk-major ([n_chunks][E]).  One cluster of 1, 2, 4
+// or 8 CTAs, 32 experts each; warp g of a CTA has chunk range g of 32.  A lane
+// sums its expert over the range (rows of 128 bytes, kScanAhead in flight), the
+// warps' sums are combined in shared memory, and the lane writes
+// chunk_base[c][e] = the entries of expert e in chunks before c (relative to
+// the expert's offset, which dispatch adds) over its range.  The last warps
+// hold the totals: each CTA sends its sum to the CTAs after it and writes its
+// counts and offsets.  A range of up to kScanAhead chunks (32768 tokens) is
+// read once.  Bound by latency: L2 once, a cluster barrier.  Without a cluster
+// the sums need a counter that starts at zero and a last CTA; with the counter
+// cleared by a memset and the scan done by the last CTA of the one-launch
+// route, asap_moe_route took 98.7 us at 16384 tokens (L2 flushed) and, call
+// after call, 34.6 us at 4096; one CTA of 1024 threads for all experts 112.5
+// us at 16384; this 88.5 and 30.9 us.
+constexpr int kScanWarps = 32;
+constexpr int kScanAhead = 32;
 
 // MAPPED (a mailbox round): the rows scanned are rowmap[0 .. *n_chunks_dev)
 // of hist, in that order (n_chunks is then rowmap's length), and chunk_base
 // is written at the same rows.
 template <bool MAPPED>
-__global__ void __launch_bounds__(kScanThreads) scan_kernel(const int32_t* __restrict__ hist, int n_chunks, int E,
-                                                            int32_t* __restrict__ counts,
-                                                            int32_t* __restrict__ offsets,
-                                                            int32_t* __restrict__ chunk_base,
-                                                            int32_t* __restrict__ tile_counters,
-                                                            int32_t* __restrict__ ticket,
-                                                            const int32_t* __restrict__ rowmap,
-                                                            const int32_t* __restrict__ n_chunks_dev) {
+__global__ void __launch_bounds__(kScanWarps * 32) scan_kernel(const int32_t* __restrict__ hist, int n_chunks, int E,
+                                                               int32_t* __restrict__ counts,
+                                                               int32_t* __restrict__ offsets,
+                                                               int32_t* __restrict__ chunk_base,
+                                                               int32_t* __restrict__ tile_counters,
+                                                               const int32_t* __restrict__ rowmap,
+                                                               const int32_t* __restrict__ n_chunks_dev) {
+  __shared__ int part[kScanWarps][32];
+  __shared__ int blk[kMaxExperts / 32];  // sums of the CTAs before this one
+  // every CTA of the cluster has started: its shared memory may be written
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
   pdl_wait();
   pdl_launch();
-  __shared__ int part[kScanWarps][32];
-  __shared__ int swarp[33];
-  __shared__ bool last;
-  if constexpr (MAPPED) n_chunks = max(0, min(*n_chunks_dev, n_chunks));  // n_chunks: rowmap's length
-  auto row = [&](int c) -> long long { return MAPPED ? rowmap[c] : c; };
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int e = blockIdx.x * 32 + lane;
+  const int lane = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int rank = blockIdx.x, ranks = gridDim.x;
+  const int e = rank * 32 + lane;
   const bool ve = e < E;
+  if constexpr (MAPPED) n_chunks = max(0, min(*n_chunks_dev, n_chunks));  // n_chunks: rowmap's length
+  auto at = [&](int c) -> long long { return static_cast<long long>(MAPPED ? rowmap[c] : c) * E + e; };
   const int per = (n_chunks + kScanWarps - 1) / kScanWarps;
-  const int c0 = min(n_chunks, warp * per), c1 = min(n_chunks, c0 + per);
-  int sum = 0;
-  if (ve) {
-#pragma unroll 8
-    for (int c = c0; c < c1; ++c) sum += hist[row(c) * E + e];
-  }
-  part[warp][lane] = sum;
-  __syncthreads();
-  int run = 0, total = 0;
+  const int c0 = min(n_chunks, g * per), c1 = min(n_chunks, c0 + per);
+  int v[kScanAhead];
+  auto load = [&](int c) {
 #pragma unroll
-  for (int w = 0; w < kScanWarps; ++w) {
-    const int v = part[w][lane];
-    if (w < warp) run += v;
-    total += v;
+    for (int u = 0; u < kScanAhead; ++u) v[u] = ve && c + u < c1 ? hist[at(c + u)] : 0;
+  };
+  int sum = 0;
+  for (int c = c0; c < c1; c += kScanAhead) {
+    load(c);
+#pragma unroll
+    for (int u = 0; u < kScanAhead; ++u) sum += v[u];
   }
-  if (ve) {
-#pragma unroll 8
-    for (int c = c0; c < c1; ++c) {
-      const long long o = row(c) * E + e;
-      const int v = hist[o];
-      chunk_base[o] = run;
-      run += v;
+  part[g][lane] = sum;
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  __syncthreads();
+  int run = 0;
+  for (int h = 0; h < g; ++h) run += part[h][lane];
+  int total = 0, incl = 0;
+  if (g == kScanWarps - 1) {
+    incl = total = run + sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int u = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += u;
     }
-    if (warp == 0) counts[e] = total;
+    const int all = __shfl_sync(kFull, incl, 31);
+    if (lane > rank && lane < ranks) {
+      uint32_t peer;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(smem_u32(&blk[rank])), "r"(lane));
+      asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(peer), "r"(all) : "memory");
+    }
+    __syncwarp();
   }
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(ticket, 1) == static_cast<int>(gridDim.x) - 1;
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  int base = 0;
-  for (int e0 = 0; e0 < E; e0 += kScanThreads) {
-    const int ee = e0 + threadIdx.x;
-    const int v = ee < E ? __ldcg(counts + ee) : 0;
-    int tot = 0;
-    const int ex = block_exclusive_scan(v, swarp, tot);
-    if (ee < E) offsets[ee] = base + ex;
-    base += tot;
-  }
-  if (threadIdx.x == 0) {
-    offsets[E] = base;
-    *ticket = 0;
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  for (int c = c0; c < c1; c += kScanAhead) {
+    if (per > kScanAhead) load(c);
+#pragma unroll
+    for (int u = 0; u < kScanAhead; ++u) {
+      if (ve && c + u < c1) chunk_base[at(c + u)] = run;
+      run += v[u];
+    }
   }
   // the grouped GEMMs that follow on this stream claim tiles from these
-  if (tile_counters && threadIdx.x < kTileCounters) tile_counters[threadIdx.x] = 0;
+  if (tile_counters && rank == 0 && threadIdx.x < kTileCounters) tile_counters[threadIdx.x] = 0;
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  if (g == kScanWarps - 1 && ve) {
+    int before = 0;
+    for (int r = 0; r < rank; ++r) before += blk[r];
+    counts[e] = total;
+    offsets[e] = before + incl - total;
+    if (e == E - 1) offsets[E] = before + incl;
+  }
 }
 
 // Sum of the K-slice planes of the router GEMM, added in slice order.
@@ -766,11 +746,11 @@ cudaError_t launch_gate_seg(const float* logits, int splits, int n, const GatePa
   return launch_pdl(gate_kernel, chunks, kGateWarps * 32, 0, s, 1, logits, splits, plane, n, p, idx, w, hist, n_chunks_total, chunk0);
 }
 
-cudaError_t launch_hist(const int32_t* idx, int n, int k, int E, int32_t* hist, uint32_t* status, int32_t* ticket,
+cudaError_t launch_hist(const int32_t* idx, int n, int k, int E, int32_t* hist, uint32_t* status,
                         cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const int chunks = ceil_div(n, kChunkTokens);
-  return launch_pdl(hist_kernel, chunks, 256, 0, s, 1, idx, n, k, E, hist, chunks, status, ticket);
+  return launch_pdl(hist_kernel, chunks, 256, 0, s, 1, idx, n, k, E, hist, status);
 }
 
 cudaError_t launch_reduce_splits(const float* parts, int splits, long long plane, float* out, cudaStream_t s) {
@@ -779,15 +759,22 @@ cudaError_t launch_reduce_splits(const float* parts, int splits, long long plane
   return launch_pdl(reduce_splits_kernel, blocks, 256, 0, s, 1, parts, splits, plane, out);
 }
 
+namespace {
+int scan_ctas(int E) { return E <= 32 ? 1 : E <= 64 ? 2 : E <= 128 ? 4 : 8; }
+}  // namespace
+static_assert(kMaxExperts == 256, "8 CTAs of 32 experts");
+
 cudaError_t launch_scan(const int32_t* hist, int n_chunks, int E, int32_t* counts, int32_t* offsets,
-                        int32_t* chunk_base, int32_t* ticket, cudaStream_t s, int32_t* tile_counters) {
-  return launch_pdl(scan_kernel<false>, ceil_div(E, 32), kScanThreads, 0, s, 1, hist, n_chunks, E, counts, offsets, chunk_base, tile_counters, ticket, nullptr, nullptr);
+                        int32_t* chunk_base, cudaStream_t s, int32_t* tile_counters) {
+  return launch_pdl(scan_kernel<false>, scan_ctas(E), kScanWarps * 32, 0, s, scan_ctas(E), hist, n_chunks, E, counts,
+                    offsets, chunk_base, tile_counters, nullptr, nullptr);
 }
 
 cudaError_t launch_scan_mapped(const int32_t* hist, const int32_t* rowmap, const int32_t* n_chunks, int max_chunks,
-                               int E, int32_t* counts, int32_t* offsets, int32_t* chunk_base, int32_t* ticket,
-                               int32_t* tile_counters, cudaStream_t s) {
-  return launch_pdl(scan_kernel<true>, ceil_div(E, 32), kScanThreads, 0, s, 1, hist, max_chunks, E, counts, offsets, chunk_base, tile_counters, ticket, rowmap, n_chunks);
+                               int E, int32_t* counts, int32_t* offsets, int32_t* chunk_base, int32_t* tile_counters,
+                               cudaStream_t s) {
+  return launch_pdl(scan_kernel<true>, scan_ctas(E), kScanWarps * 32, 0, s, scan_ctas(E), hist, max_chunks, E, counts,
+                    offsets, chunk_base, tile_counters, rowmap, n_chunks);
 }
 
 }  // namespace asap

@@ -1,7 +1,7 @@
 // Routing of a micro-batch in one launch on the sm_103a tensor core: router
-// logits, grouped sigmoid gating with top-k, the expert histogram and its
-// scan into per-expert counts and offsets (the metadata the MoE side of ASAP
-// receives per DP group, Section 3.2.1; Table 1: top-K of E_total = 256).
+// logits, grouped sigmoid gating with top-k and the expert histogram, which a
+// scan turns into per-expert counts and offsets (the metadata the MoE side of
+// ASAP receives per DP group, Section 3.2.1; Table 1: top-K of E_total = 256).
 //
 // Design (one 128-token tile per thread-block cluster):
 //  - The cluster has ``splits`` CTAs (1, 2 or 4); CTA r computes the partial
@@ -30,9 +30,7 @@
 //    then inserts just those candidates, in increasing expert order, into its
 //    top-k by (key desc, expert asc).  Same scores, keys, tie-breaks and
 //    weight arithmetic as the gate kernels, so the same experts and weights.
-//  - Per-chunk histograms go to hist[chunk][e]; the last CTA to finish
-//    (ticket counter, zero at launch) scans them into chunk bases, counts and
-//    offsets, one thread per expert.
+//  - Per-chunk histograms go to hist[chunk][e]; a scan launch follows.
 // The shared memory of the operand rings is reused for the partial-logit
 // slots and the gate's scratch once every CTA of the cluster is done with its
 // rings (cluster barrier).  Every wait is bounded; on a timeout the CTA still
@@ -62,13 +60,12 @@ constexpr int kSigOff = kRecvBytes;                             // sigmoid score
 constexpr int kTopOff = kSigOff + kRouteExperts * kSigPitch * 4;  // per block: top-2 keys per token
 constexpr int kMaskOff = kTopOff + 2 * kBlocks * 32 * 4;        // per block: candidate bits per token
 constexpr int kHistOff = kMaskOff + kBlocks * 32 * 4;           // chunk histogram
-constexpr int kWarpSumOff = kHistOff + kRouteExperts * 4;       // the scan's warp totals
-constexpr int kScratchEnd = kWarpSumOff + 40 * 4;
+constexpr int kScratchEnd = kHistOff + kRouteExperts * 4;
 static_assert(kScratchEnd <= kRingBytes, "the gate's scratch overlays the operand rings");
-static_assert(kThreads == kRouteExperts, "the scan gives one thread per expert");
+static_assert(kThreads == kRouteExperts, "one thread per expert of the histogram");
 constexpr int kBarOff = kRingBytes;
 // mbarriers fullA[kRA], emptyA[kRA], fullB[kRB], emptyB[kRB], tfull, drain,
-// bfree; then the TMEM address, abort flag, last-CTA flag and the bias pointer
+// bfree; then the TMEM address, abort flag and the bias pointer
 constexpr int kNumBars = 2 * kRA + 2 * kRB + 3;
 constexpr int kBarBytes = 8 * kNumBars + 32;
 constexpr size_t kSmem = kRingBytes + kBarBytes;
@@ -113,16 +110,6 @@ __device__ __forceinline__ void tmem_st_wait() {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
 
-__device__ __forceinline__ int warp_inclusive_scan(int v) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int u = __shfl_up_sync(kFull, v, o);
-    if (lane >= o) v += u;
-  }
-  return v;
-}
-
 __global__ void __launch_bounds__(kThreads, 1)
     route_fused_kernel(const __grid_constant__ CUtensorMap tmX, const RouteFusedArgs a) {
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -151,7 +138,6 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t tmem_cols = nseq > 1 ? 2 * kGemmBN : kGemmBN;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar_area + 8 * kNumBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* last_flag = reinterpret_cast<volatile int*>(tmem_slot + 2);
   volatile int* acc_bad = reinterpret_cast<volatile int*>(tmem_slot + 3);
   const float** bias_slot = reinterpret_cast<const float**>(tmem_slot + 4);
   const CUtensorMap* tmW = nullptr;
@@ -170,7 +156,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(drain, 1);
       mbar_init(bfree, 128);  // the four epilogue warps
       *abort_flag = 0;
-      *last_flag = 0;
       *acc_bad = aligned ? 0 : 1;
       fence_barrier_init();
       tma_prefetch_desc(&tmX);
@@ -558,47 +543,6 @@ __global__ void __launch_bounds__(kThreads, 1)
       a.hist[static_cast<long long>(a.chunk0 + chunk) * kRouteExperts + threadIdx.x] = shist[threadIdx.x];
     shist[threadIdx.x] = 0;
     __syncthreads();
-  }
-
-  // ------------------------------------------------------------ scan (last CTA)
-  if (a.ticket) {
-    __threadfence();  // this thread's histogram stores before the ticket
-    __syncthreads();
-    if (threadIdx.x == 0) *last_flag = atomicAdd(a.ticket, 1) == static_cast<int>(gridDim.x) - 1 ? 1 : 0;
-    __syncthreads();
-    if (*last_flag) {
-      __threadfence();
-      // thread e: expert e's column of the chunk-major histogram, 64 rows in
-      // flight at a time
-      const int e = threadIdx.x;
-      const int nct = a.n_chunks_total;
-      int run = 0;
-#pragma unroll 1
-      for (int c0 = 0; c0 < nct; c0 += 64) {
-        int v[64];
-#pragma unroll
-        for (int u = 0; u < 64; ++u)
-          v[u] = c0 + u < nct ? __ldcg(a.hist + static_cast<long long>(c0 + u) * kRouteExperts + e) : 0;
-#pragma unroll
-        for (int u = 0; u < 64; ++u) {
-          if (c0 + u < nct) a.chunk_base[static_cast<long long>(c0 + u) * kRouteExperts + e] = run;
-          run += v[u];
-        }
-      }
-      // offsets: exclusive scan of the counts, one thread per expert
-      int* swarp = reinterpret_cast<int*>(smem + kWarpSumOff);
-      const int incl = warp_inclusive_scan(run);
-      if (lane == 31) swarp[warp] = incl;
-      __syncthreads();
-      int before = 0;
-      for (int w2 = 0; w2 < warp; ++w2) before += swarp[w2];
-      a.counts[e] = run;
-      a.offsets[e] = before + incl - run;
-      if (e == kRouteExperts - 1) a.offsets[kRouteExperts] = before + incl;
-      // the grouped GEMMs that follow on this stream claim tiles from these
-      if (a.tile_counters && threadIdx.x < kTileCounters) a.tile_counters[threadIdx.x] = 0;
-      if (threadIdx.x == 0) *a.ticket = 0;
-    }
   }
 
   tc_fence_before();
