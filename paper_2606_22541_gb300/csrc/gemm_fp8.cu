@@ -11,9 +11,9 @@
 //
 // A tile is up to 128 token rows of one expert (M) and the 256 weight rows of
 // an n-tile (N), on one SM: handing a partial between the SMs of a CTA pair
-// costs more than the operand reads that a pair saves (tokens on M over a pair:
-// 3100 instead of 2615 us for the layer of 4096 tokens; weights on M, with the
-// token scales through shared memory: 4005).  Every 128-wide K block has one of
+// costs more than the operand reads that a pair saves (with 32-column
+// chunks, the layer of 4096 tokens: tokens on M over a pair 3100 instead of
+// 2615 us; weights on M, with the token scales through shared memory, 4005).  Every 128-wide K block has one of
 // two 256-column partials.
 //
 // Roles (one CTA per SM, persistent, 384 threads):
@@ -24,16 +24,23 @@
 //   warp 3 : tile scheduler, one decoded tile ahead
 //   warps 4-11: epilogue; warp w owns TMEM lanes 32 (w % 4) .. (tokens) and one
 //            half of the columns; its warpgroups take registers from the first
-//            (56 + 2 x 224 a thread), for two 32-column chunks in flight
-//            beside 128 accumulators
+//            (56 + 2 x 224 a thread): 128 accumulators, two 16-column chunks
 // Tile schedule, masking and bounded waits as in the bf16 kernels.
 //
 // What bounds it (DeepSeek-V3 shape, Zipf routing, gate/up | down us of one
 // call; before: roles issuing from lanes that had left their warps, every role
-// decoding its tiles, 16 columns per TMEM wait): 128 tokens 661 | 334 (684 |
-// 348), the weight stream; 4096 tokens 1525 | 863 (1778 | 1024) and 16384
-// tokens 3883 | 2363 (4730 | 2796): 48 KB of operands per K block from L2, and
-// the promotion (without it 4096 tokens take 1450 | 815, 16384 3349 | 1970).
+// decoding its tiles, 16 columns per TMEM wait): 128 tokens 576 | 292 (684 |
+// 348), the weight stream; 4096 tokens 1435 | 786 (1778 | 1024) and 16384
+// tokens 3650 | 2170 (4730 | 2796): the operands (48 KB per K block through L2
+// and shared memory; with every second box left out 4096 tokens take 1231 |
+// 687 and 16384 3267 | 1934) and the promotion (with a quarter of it 1412 | 747
+// and 3279 | 1844).  In the promotion a 16-column chunk is on its way from TMEM
+// while the one before it is added: 4096 tokens took 1469 | 821 with chunks of
+// 32 and two on their way or none, which spill in either order (in the order
+// used here 2224 | 1148); the row scales as 16-byte loads of four K blocks
+// (moves and a branch per K block) 1560 | 851; looking at the next partial's
+// barrier ahead 1437 | 788.  Weights prefetched into L2 4, 8 or 16 K blocks
+// ahead: 1519, 1532 and 1553 for gate/up.
 #include "common.cuh"
 #include "gemm_config.h"
 #include "gemm_sched.cuh"
@@ -88,9 +95,9 @@ __device__ __forceinline__ void tc_mma_f8(uint32_t d_tmem, uint64_t adesc, uint6
       : "memory");
 }
 
-__device__ __forceinline__ void add32(float* acc, const uint32_t (&v)[32], float s) {
+__device__ __forceinline__ void add16(float* acc, const uint32_t (&v)[16], float s) {
 #pragma unroll
-  for (int j = 0; j < 32; ++j) acc[j] = fmaf(s, __uint_as_float(v[j]), acc[j]);
+  for (int j = 0; j < 16; ++j) acc[j] = fmaf(s, __uint_as_float(v[j]), acc[j]);
 }
 
 // One round of a warp's coalesced stores: lane l holds 4 chunks of 16 bytes
@@ -318,12 +325,42 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int layer = *layer_slot;
     Ring<kSlots> p;
     bool ok = true;
-    PairTile T;
-    for (int it = 0; ok; ++it) {
-      ok = __all_sync(0xffffffffu, tq.pop(T, abort_flag));
-      if (!ok) break;
+    PairTile T, next;
+    // the scales of a tile's first two K blocks are loaded (L2 latency) before
+    // the tile in front of it is written, the others two K blocks ahead
+    float a0 = 0.f, l0 = 0.f, h0 = 0.f, a1 = 0.f, l1 = 0.f, h1 = 0.f;
+    const float *arow = nullptr, *bs_lo = nullptr, *bs_hi = nullptr;
+    auto ld_scales = [&](int kb, int k_iters, float& a, float& bl, float& bh) {
+      if (kb < k_iters) {
+        a = __ldg(arow + kb);
+        bl = __ldg(bs_lo + kb);
+        bh = EPI == EPI_SWIGLU ? __ldg(bs_hi + kb) : 0.f;
+      }
+    };
+    auto pop_next = [&]() -> bool {
+      const bool got = __all_sync(0xffffffffu, tq.pop(next, abort_flag));
+      if (!got) return false;
       if (lane == 0) tq.release();
       ++tq.n;
+      const int valid = next.rows - q * 32;
+      if (next.k_iters == 0 || valid <= 0) return true;
+      const int sld = next.p1 ? fa.a_sld1 : fa.a_sld0;
+      arow = (next.p1 ? fa.a_scale1 : fa.a_scale0) +
+             (static_cast<long long>(next.row) + q * 32 + min(lane, valid - 1)) * sld;  // masked rows: the last valid one
+      // scale rows of this warp's columns: SwiGLU tiles hold gate block nt
+      // (scale row 2 nt) and up block nt (2 nt + 1); plain tiles blocks 2 nt, 2 nt + 1
+      bs_lo = args.lref.table[layer].scale[next.p1 ? args.bmap1 : args.bmap0] +
+              (static_cast<long long>(next.group) * (next.p1 ? fa.b_nblk1 : fa.b_nblk0) + 2 * next.n_tile +
+               (EPI == EPI_SWIGLU ? 0 : cq)) *
+                  sld;
+      bs_hi = bs_lo + sld;
+      ld_scales(0, next.k_iters, a0, l0, h0);
+      ld_scales(1, next.k_iters, a1, l1, h1);
+      return true;
+    };
+    ok = pop_next();
+    for (int it = 0; ok; ++it) {
+      T = next;
       if (T.k_iters == 0) break;
       const int valid_rows = T.rows - q * 32;  // rows of this warp
       const long long row = static_cast<long long>(T.row) + r;
@@ -335,63 +372,64 @@ __global__ void __launch_bounds__(kThreads, 1)
           p.advance();
         }
         if (EPI == EPI_SWIGLU && ok) mbar_arrive(bar(B_XC, it & 1));
+        ok = ok && pop_next();
         continue;
       }
-      const int sld = T.p1 ? fa.a_sld1 : fa.a_sld0;
-      const float* arow = (T.p1 ? fa.a_scale1 : fa.a_scale0) +
-                          (lane < valid_rows ? row : row - lane + valid_rows - 1) * sld;  // masked rows: the last valid one
-      // scale rows of this warp's columns: SwiGLU tiles hold gate block nt
-      // (scale row 2 nt) and up block nt (2 nt + 1); plain tiles blocks 2 nt, 2 nt + 1
-      const float* bs_lo = args.lref.table[layer].scale[T.p1 ? args.bmap1 : args.bmap0] +
-                           (static_cast<long long>(T.group) * (T.p1 ? fa.b_nblk1 : fa.b_nblk0) + 2 * T.n_tile +
-                            (EPI == EPI_SWIGLU ? 0 : cq)) *
-                               sld;
-      const float* bs_hi = bs_lo + sld;
-      // scales of the next two K blocks are loaded ahead (L2 latency)
-      auto ld_scales = [&](int kb, float& a, float& bl, float& bh) {
-        if (kb < T.k_iters) {
-          a = __ldg(arow + kb);
-          bl = __ldg(bs_lo + kb);
-          bh = EPI == EPI_SWIGLU ? __ldg(bs_hi + kb) : 0.f;
-        }
-      };
-      float a0 = 0.f, l0 = 0.f, h0 = 0.f, a1 = 0.f, l1 = 0.f, h1 = 0.f;
-      ld_scales(0, a0, l0, h0);
-      ld_scales(1, a1, l1, h1);
       float acc[kCols];
 #pragma unroll
       for (int j = 0; j < kCols; ++j) acc[j] = 0.f;
+      uint32_t c0[16], c1[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) c1[j] = 0u;
+      float s_prev = 0.f;
       for (int kb = 0; kb < T.k_iters; ++kb) {
         const float s_lo = a0 * l0;
         const float s_hi = EPI == EPI_SWIGLU ? a0 * h0 : s_lo;
         a0 = a1;
         l0 = l1;
         h0 = h1;
-        ld_scales(kb + 2, a1, l1, h1);
+        ld_scales(kb + 2, T.k_iters, a1, l1, h1);
         if (!__all_sync(0xffffffffu, mbar_wait(bar(B_PF, p.s), p.phase, abort_flag))) {
           ok = false;
           break;
         }
         tc_fence_after();
-        // four chunks of 32 columns, two in flight; the partial is handed back
-        // when the last two are in registers
+        // eight chunks of 16 columns: one is on its way from TMEM while the
+        // one before it is added, across K blocks too; the partial is handed
+        // back when its last chunk is in registers
         const uint32_t ta = col + p.s * 256;
-        uint32_t c0[32], c1[32];
-        tmem_ld32(ta, c0);
-        tmem_ld32(ta + 32, c1);
+        tmem_ld16(ta, c0);
+        add16(acc + 112, c1, s_prev);
         tmem_ld_wait();
-        add32(acc, c0, s_lo);
-        tmem_ld32(ta + kHi, c0);
-        add32(acc + 32, c1, s_lo);
-        tmem_ld32(ta + kHi + 32, c1);
+        tmem_ld16(ta + 16, c1);
+        add16(acc + 0, c0, s_lo);
+        tmem_ld_wait();
+        tmem_ld16(ta + 32, c0);
+        add16(acc + 16, c1, s_lo);
+        tmem_ld_wait();
+        tmem_ld16(ta + 48, c1);
+        add16(acc + 32, c0, s_lo);
+        tmem_ld_wait();
+        tmem_ld16(ta + kHi, c0);
+        add16(acc + 48, c1, s_lo);
+        tmem_ld_wait();
+        tmem_ld16(ta + kHi + 16, c1);
+        add16(acc + 64, c0, s_hi);
+        tmem_ld_wait();
+        tmem_ld16(ta + kHi + 32, c0);
+        add16(acc + 80, c1, s_hi);
+        tmem_ld_wait();
+        tmem_ld16(ta + kHi + 48, c1);
+        add16(acc + 96, c0, s_hi);
         tmem_ld_wait();
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(bar(B_PE, p.s));
-        add32(acc + 64, c0, s_hi);
-        add32(acc + 96, c1, s_hi);
+        s_prev = s_hi;
         p.advance();
       }
+      add16(acc + 112, c1, s_prev);
+      ok = ok && pop_next();
       if (!ok) break;
       const long long wrow0 = row - lane;
       if constexpr (EPI == EPI_SWIGLU) {
