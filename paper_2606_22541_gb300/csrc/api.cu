@@ -277,10 +277,9 @@ int run_gate_scan(asap_moe_t h, const float* logits, int splits, int n, int32_t*
   const Layout L = layout(h->cfg, n);
   int32_t* hist = at<int32_t>(ws, L.hist);
   int32_t* base = at<int32_t>(ws, L.chunk_base);
-  CU_TRY(asap::launch_gate(logits, splits, n, gate_params(h, layer), idx, w, hist, st), "gate launch");
-  CU_TRY(asap::launch_scan(hist, asap::ceil_div(n, asap::kChunkTokens), h->cfg.n_experts, counts, offsets, base, st,
-                           at<int32_t>(ws, L.tile_counters)),
-         "scan launch");
+  CU_TRY(asap::launch_gate_scan(logits, splits, n, gate_params(h, layer), idx, w, hist, counts, offsets, base,
+                                at<int32_t>(ws, L.tile_counters), st),
+         "gate and scan launch");
   return ASAP_OK;
 }
 
@@ -940,14 +939,13 @@ ASAP_API int asap_moe_dispatch(asap_moe_t h, const void* x, int32_t n, const int
   if (h->fp8 && !x_perm_scales) return fail(ASAP_ERR_INVALID, "the FP8 configuration needs x_perm_scales");
   const asap_moe_config& c = h->cfg;
   const Layout L = layout(c, n);
-  const int chunks = asap::ceil_div(n, asap::kChunkTokens);
   cudaStream_t st = S(stream);
   int32_t* hist = at<int32_t>(ws, L.hist);
   int32_t* base = at<int32_t>(ws, L.chunk_base);
   int32_t* offs = at<int32_t>(ws, L.offsets);
-  CU_TRY(asap::launch_hist(idx, n, c.top_k, c.n_experts, hist, h->status, st), "hist launch");
-  CU_TRY(asap::launch_scan(hist, chunks, c.n_experts, at<int32_t>(ws, L.counts), offs, base, st),
-         "scan launch");
+  CU_TRY(asap::launch_hist_scan(idx, n, c.top_k, c.n_experts, hist, at<int32_t>(ws, L.counts), offs, base, h->status,
+                                st),
+         "histogram and scan launch");
   if (h->fp8)
     CU_TRY(asap::launch_dispatch_fp8(x, n, c.hidden, c.top_k, c.n_experts, idx, base, offs, x_perm, x_perm_scales,
                                      nullptr, nullptr, perm_src, perm_dst, h->status, st),
@@ -1782,15 +1780,12 @@ ASAP_API int asap_moe_route_noalloc(asap_moe_t h, const void* x, int32_t n, int3
   int32_t* hist = reinterpret_cast<int32_t*>(scratch + kStaticLogitsBytes);
   int32_t* base = reinterpret_cast<int32_t*>(scratch + kStaticLogitsBytes + kStaticChunkBytes);
   cudaStream_t st = S(stream);
-  auto scan = [&]() -> int {
-    CU_TRY(asap::launch_scan(hist, asap::ceil_div(n, asap::kChunkTokens), h->cfg.n_experts, counts, offsets, base, st),
-           "scan launch");
-    return ASAP_OK;
-  };
   if (fused_route(h)) {
     // the same launches as asap_moe_route (same K slices, same bits)
     if ((r = run_route_fused(h, x, n, idx, w, hist, 0, h->layer_ids, st)) != ASAP_OK) return r;
-    return scan();
+    CU_TRY(asap::launch_scan(hist, asap::ceil_div(n, asap::kChunkTokens), h->cfg.n_experts, counts, offsets, base, st),
+           "scan launch");
+    return ASAP_OK;
   }
   // the router's K slices and their order of addition are those of
   // asap_moe_route, so the bits are the same.  Every scratch element read
@@ -1799,6 +1794,8 @@ ASAP_API int asap_moe_route_noalloc(asap_moe_t h, const void* x, int32_t n, int3
   // nothing has to be cleared between calls.
   const int splits = router_splits(h, n);
   if ((r = run_router_logits(h, x, n, logits, splits, h->layer_ids, st)) != ASAP_OK) return r;
-  CU_TRY(asap::launch_gate(logits, splits, n, gate_params(h, h->layer_ids), idx, w, hist, st), "gate launch");
-  return scan();
+  CU_TRY(asap::launch_gate_scan(logits, splits, n, gate_params(h, h->layer_ids), idx, w, hist, counts, offsets, base,
+                                nullptr, st),
+         "gate and scan launch");
+  return ASAP_OK;
 }

@@ -184,9 +184,14 @@ cudaError_t launch_reduce_splits(const float* parts, int splits, long long plane
 // n_chunks_total rows.
 cudaError_t launch_gate_seg(const float* logits, int splits, int n, const GateParams& p, int32_t* idx, float* w,
                             int32_t* hist, int chunk0, int n_chunks_total, cudaStream_t s);
-// hist as launch_gate writes it.
-cudaError_t launch_hist(const int32_t* idx, int n, int k, int E, int32_t* hist, uint32_t* status,
-                        cudaStream_t s);
+// launch_gate and launch_scan of its histogram (hist: scratch that a call of few
+// chunks does not write).
+cudaError_t launch_gate_scan(const float* logits, int splits, int n, const GateParams& p, int32_t* idx, float* w,
+                             int32_t* hist, int32_t* counts, int32_t* offsets, int32_t* chunk_base,
+                             int32_t* tile_counters, cudaStream_t s);
+// The histogram of idx and its scan (hist: scratch for large calls).
+cudaError_t launch_hist_scan(const int32_t* idx, int n, int k, int E, int32_t* hist, int32_t* counts,
+                             int32_t* offsets, int32_t* chunk_base, uint32_t* status, cudaStream_t s);
 // counts, offsets, and chunk_base[c][e] = entries of expert e in chunks
 // before c (relative: the absolute base is offsets[e] + chunk_base[c][e]);
 // hist and chunk_base are chunk-major [n_chunks][E].

@@ -1,5 +1,7 @@
-"""Dispatch's histogram scan over chunk ranges of one, two and several loads and
-one to eight blocks of 32 experts: offsets and positions against a stable sort."""
+"""The histogram and scan of dispatch, by one cluster (up to 8192 tokens) and by
+a launch each, over chunk ranges of every kind and one to eight blocks of 32
+experts, against a stable sort; the scan of the gate (by the gate's own cluster
+up to 256 tokens) against a count and against dispatch."""
 import pytest
 import torch
 
@@ -11,7 +13,7 @@ DEV = "cuda:0"
 
 
 @pytest.mark.parametrize("experts", [1, 32, 33, 100, 256])
-@pytest.mark.parametrize("n", [1, 33, 1025, 32769, 66000])
+@pytest.mark.parametrize("n", [1, 33, 65, 1025, 8192, 8193, 32769, 66000])
 def test_scan(experts, n):
     k = min(2, experts)
     cfg = inputs.small_variant(MIXTRAL, name="scan", hidden=256, inter=256, n_experts=experts, top_k=k, seed=5)
@@ -32,3 +34,33 @@ def test_scan(experts, n):
     assert torch.equal(dst.flatten().long()[order], torch.arange(n * k, device=DEV))
     assert torch.equal(src.long(), order // k)
     assert torch.equal(xp, x[order // k])
+
+
+@pytest.mark.parametrize("experts", [8, 16, 24, 32, 64, 128, 256])
+@pytest.mark.parametrize("n", [1, 32, 33, 65, 129, 255, 256, 257])
+def test_gate_scan(experts, n):
+    cfg = inputs.small_variant(MIXTRAL, name="gate", hidden=256, inter=256, n_experts=experts, top_k=2, seed=6)
+    h = api.asap_moe_create(cfg, inputs.make_weights(cfg, DEV), n)
+    x = inputs.make_tokens(cfg, n, 0, DEV)
+    ws = api.workspace(h, n)
+    i32 = dict(dtype=torch.int32, device=DEV)
+    idx, w = torch.empty((n, 2), **i32), torch.empty((n, 2), device=DEV)
+    counts, offs = torch.empty(experts, **i32), torch.empty(experts + 1, **i32)
+    for _ in range(2):
+        counts.fill_(-1), offs.fill_(-1)
+        api.asap_moe_route(h, x, idx, w, counts, offs, ws)
+    want = torch.bincount(idx.flatten().long(), minlength=experts)
+    assert torch.equal(counts.long(), want)
+    assert torch.equal(offs.long(), torch.cat([want.new_zeros(1), want.cumsum(0)]))
+    # the layer's positions (from the gate's scan) and dispatch's give the same output
+    out = torch.empty_like(x)
+    api.asap_moe_layer(h, x, out, ws)
+    xp = torch.empty((2 * n, cfg.hidden), dtype=torch.bfloat16, device=DEV)
+    src, dst = torch.empty(2 * n, **i32), torch.empty((n, 2), **i32)
+    y = torch.empty_like(xp)
+    step = torch.empty_like(x)
+    api.asap_moe_dispatch(h, x, idx, xp, src, dst, ws)
+    api.asap_moe_expert_ffn(h, xp, offs, x, y, None, ws)
+    api.asap_moe_combine(h, y, None, w, dst, step)
+    assert api.asap_moe_status(h) == (0, 0)
+    assert torch.equal(out.view(torch.int16), step.view(torch.int16))
