@@ -37,7 +37,7 @@ def test_scan(experts, n):
 
 
 @pytest.mark.parametrize("experts", [8, 16, 24, 32, 64, 128, 256])
-@pytest.mark.parametrize("n", [1, 32, 33, 65, 129, 255, 256, 257])
+@pytest.mark.parametrize("n", [1, 17, 32, 33, 65, 129, 255, 256, 257])
 def test_gate_scan(experts, n):
     cfg = inputs.small_variant(MIXTRAL, name="gate", hidden=256, inter=256, n_experts=experts, top_k=2, seed=6)
     h = api.asap_moe_create(cfg, inputs.make_weights(cfg, DEV), n)
