@@ -250,8 +250,9 @@ def sources_sha256(files):
     return d.hexdigest()
 
 
-GEMM_SOURCES = ["paper_2606_22541_gb300/csrc/gemm_tc.cu", "paper_2606_22541_gb300/csrc/common.cuh",
-                "paper_2606_22541_gb300/csrc/gemm_sched.cuh", "paper_2606_22541_gb300/csrc/gemm_config.h"]
+GEMM_SOURCES = ["paper_2606_22541_gb300/csrc/gemm_pair.cu", "paper_2606_22541_gb300/csrc/pair.cuh",
+                "paper_2606_22541_gb300/csrc/common.cuh", "paper_2606_22541_gb300/csrc/gemm_sched.cuh",
+                "paper_2606_22541_gb300/csrc/gemm_config.h"]
 
 
 def weight_gb(cfg):
@@ -333,11 +334,13 @@ def run_ours(args, dist):
     code, word = api.asap_moe_status(h)
     if code != 0:
         raise RuntimeError(f"device status word {word:#x} after the timed region")
-    # route (one kernel for E = 256 with grouped sigmoid gating, else router,
-    # gate and scan), dispatch, gate/up GEMM, down GEMM, combine (none when
-    # the combine runs inside the down GEMM)
+    # route (router with gate, then scan, for E = 256 with grouped sigmoid gating;
+    # else router, gate and scan, the latter two in one up to 256 tokens),
+    # dispatch, gate/up GEMM, down GEMM, combine (none when the combine runs
+    # inside the down GEMM)
     fused = cfg.n_experts == 256 and cfg.gating == "sigmoid_grouped" and cfg.n_groups in (1, 2, 4, 8)
-    launches_per_mb = (1 if fused else 3) + (3 if args.fused_combine and cfg.dtype == "bf16" else 4)
+    launches_per_step = sum((2 if fused or n <= 256 else 3) + (3 if args.fused_combine and cfg.dtype == "bf16" else 4)
+                            for n in mbs)
     result = {
         "metric": METRIC,
         "value": dist.world * tokens_per_step * args.steps / (elapsed_ms / 1e3),
@@ -359,7 +362,7 @@ def run_ours(args, dist):
                    "parallelism": f"replicas x{dist.world} (no data-path collective)",
                    "l2": f"inputs larger than L2: {weight_gb(cfg):.1f} GB of expert weights streamed every step",
                    **({"combine": "fused into the down GEMM"} if args.fused_combine and cfg.dtype == "bf16" else {})},
-        "gpu_launches": launches_per_mb * len(mbs) * args.steps,
+        "gpu_launches": launches_per_step * args.steps,
         "clocks": clk,
     }
 
