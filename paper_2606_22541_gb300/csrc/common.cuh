@@ -61,8 +61,39 @@ __device__ __forceinline__ float gate_sigmoid(float l) { return __fdividef(1.0f,
 // waits so, all kernels before that one).  pdl_launch allows the next kernel to
 // start once every CTA has called it or left.  The small kernels call it when
 // their own wait is over, the GEMMs when a CTA has no tiles left.
+//
+// Such a kernel is resident while the data it will read is still being written,
+// so nothing an earlier kernel or the caller writes is read-only for its
+// lifetime: it is read with ld_dep or a plain load, never with __ldg or through
+// a const __restrict__ pointer (the non-coherent path, whose loads may also be
+// moved above pdl_wait).  __ldg is for the weights, their scales and the
+// router's bias.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Coherent load that stays behind pdl_wait (volatile) but may pass this
+// kernel's own plain stores (no memory clobber): of data this kernel does not
+// write.
+__device__ __forceinline__ int ld_dep(const int* p) {
+  int v;
+  asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ld_dep(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 ld_dep(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint4 ld_dep(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
 
 // ---------------------------------------------------------------- smem / timers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {

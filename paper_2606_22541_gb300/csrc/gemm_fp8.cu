@@ -183,6 +183,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
   if (base & 1023u) {  // uniform for the CTA: nothing is initialised yet
+    pdl_wait();
     if (threadIdx.x == 0) record_status(args.status, ST_SMEM_ALIGN);
     return;
   }
@@ -332,7 +333,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const float *arow = nullptr, *bs_lo = nullptr, *bs_hi = nullptr;
     auto ld_scales = [&](int kb, int k_iters, float& a, float& bl, float& bh) {
       if (kb < k_iters) {
-        a = __ldg(arow + kb);
+        a = ld_dep(arow + kb);
         bl = __ldg(bs_lo + kb);
         bh = EPI == EPI_SWIGLU ? __ldg(bs_hi + kb) : 0.f;
       }

@@ -247,6 +247,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
   if (base & 1023u) {  // the same in both CTAs: nothing is initialised yet
+    pdl_wait();
     if (threadIdx.x == 0) record_status(args.status, ST_SMEM_ALIGN);
     return;
   }

@@ -141,7 +141,7 @@ __device__ __forceinline__ void decode_tile(int t, const Sched* s, int G, int to
 // the rows are reported in the status word and leave problem 0 empty.
 template <int BMT = kGemmBM>
 __device__ __forceinline__ void build_schedule(const GemmArgs& args, Sched* sch, int G, int lane) {
-  if (lane == 0) sch->m1 = args.m1_dev ? min(max(__ldg(args.m1_dev), 0), args.m1) : args.m1;
+  if (lane == 0) sch->m1 = args.m1_dev ? min(max(ld_dep(args.m1_dev), 0), args.m1) : args.m1;
   int local = 0;
   int cnt[8];
   int lo[8];
@@ -154,8 +154,8 @@ __device__ __forceinline__ void build_schedule(const GemmArgs& args, Sched* sch,
     if (g < G) {
       int m = args.m0;
       if (args.offsets) {
-        lo[i] = __ldg(args.offsets + g);
-        const int hi = __ldg(args.offsets + g + 1);
+        lo[i] = ld_dep(args.offsets + g);
+        const int hi = ld_dep(args.offsets + g + 1);
         m = hi - lo[i];
         bad |= lo[i] < 0 || m < 0 || hi > args.m0;
       }
@@ -189,14 +189,14 @@ __device__ __forceinline__ void build_schedule(const GemmArgs& args, Sched* sch,
   }
   if (lane == 31) {
     sch->tile_start[G] = incl;
-    sch->row_base[G] = args.offsets ? __ldg(args.offsets + G) : args.m0;
+    sch->row_base[G] = args.offsets ? ld_dep(args.offsets + G) : args.m0;
   }
 }
 
 // MixSched for tiles of at most MAXR rows (one full warp).
 template <int MAXR>
 __device__ __forceinline__ void build_mix_schedule(const GemmArgs& args, MixSched* sch, int G, int lane) {
-  if (lane == 0) sch->m1 = args.m1_dev ? min(max(__ldg(args.m1_dev), 0), args.m1) : args.m1;
+  if (lane == 0) sch->m1 = args.m1_dev ? min(max(ld_dep(args.m1_dev), 0), args.m1) : args.m1;
   int lo[8], m[8];
   bool bad = false;
   int nc = 0, nh = 0, tc = 0, th = 0;  // this lane's cold / hot groups and tiles
@@ -206,8 +206,8 @@ __device__ __forceinline__ void build_mix_schedule(const GemmArgs& args, MixSche
     lo[i] = 0;
     m[i] = 0;
     if (g < G) {
-      lo[i] = __ldg(args.offsets + g);
-      const int hi = __ldg(args.offsets + g + 1);
+      lo[i] = ld_dep(args.offsets + g);
+      const int hi = ld_dep(args.offsets + g + 1);
       m[i] = hi - lo[i];
       bad |= lo[i] < 0 || m[i] < 0 || hi > args.m0;
       const int mt = (max(m[i], 0) + MAXR - 1) / MAXR;
@@ -258,7 +258,7 @@ __device__ __forceinline__ void build_mix_schedule(const GemmArgs& args, MixSche
   }
   if (lane == 31) {
     sch->tile_start[G] = cold + ith;
-    sch->row_base[G] = __ldg(args.offsets + G);
+    sch->row_base[G] = ld_dep(args.offsets + G);
     sch->cold = cold;
   }
 }

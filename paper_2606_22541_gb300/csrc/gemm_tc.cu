@@ -191,7 +191,7 @@ __device__ __forceinline__ void combine_slices(const Tile& T, const GemmArgs& a,
   int t = -1;
   if (lane < valid_rows) {
     const long long r = r0 + lane;
-    t = T.p1 ? static_cast<int>(r) : __ldg(a.comb_src + r);
+    t = T.p1 ? static_cast<int>(r) : ld_dep(a.comb_src + r);
     if (t < 0 || t >= a.comb_n) {
       record_status(a.status, ST_BAD_POSITION);
       t = -1;
@@ -221,7 +221,7 @@ __device__ __forceinline__ void combine_slices(const Tile& T, const GemmArgs& a,
       wj[j] = 0.f;
       if (j < a.comb_k) {
         p[j] = __ldcg(a.comb_dst + tk + j);
-        wj[j] = __ldg(a.comb_w + tk + j);
+        wj[j] = ld_dep(a.comb_w + tk + j);
         if (p[j] < 0 || p[j] >= a.m0) {
           if (lane == 0) record_status(a.status, ST_BAD_POSITION);
           p[j] = -1;
@@ -348,6 +348,7 @@ __global__ void __launch_bounds__(Gemm<EPI, PAIR>::kThreads, 1)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t base = smem_u32(smem_raw);
   if (base & 1023u) {  // uniform for the CTA: nothing is initialised yet
+    pdl_wait();
     if (threadIdx.x == 0) record_status(args.status, ST_SMEM_ALIGN);
     return;
   }

@@ -85,7 +85,7 @@ __device__ __forceinline__ void dispatch_token(const DispatchTok& d, int V, int 
   uint4 a[kDispatchAhead];
 #pragma unroll
   for (int i = 0; i < kDispatchAhead; ++i)
-    if (tid + i * kDispatchThreads < V) a[i] = __ldg(d.x + tid + i * kDispatchThreads);
+    if (tid + i * kDispatchThreads < V) a[i] = ld_dep(d.x + tid + i * kDispatchThreads);
   const int first = d.tl * k;  // the token's first entry in the chunk
   int e = -1, at = 0;          // thread j < k: entry j's expert and its segment's position for this chunk
   if (tid < k) {
@@ -128,7 +128,7 @@ __device__ __forceinline__ void dispatch_token(const DispatchTok& d, int V, int 
     if (v0 != tid) {
 #pragma unroll
       for (int i = 0; i < kDispatchAhead; ++i)
-        if (v0 + i * kDispatchThreads < V) a[i] = __ldg(d.x + v0 + i * kDispatchThreads);
+        if (v0 + i * kDispatchThreads < V) a[i] = ld_dep(d.x + v0 + i * kDispatchThreads);
     }
 #pragma unroll
     for (int i = 0; i < kDispatchAhead; ++i) {
@@ -165,8 +165,8 @@ __device__ __forceinline__ void dispatch_token(const DispatchTok& d, int V, int 
 
 template <bool FP8>
 __global__ void __launch_bounds__(kDispatchThreads)
-    dispatch_kernel(const uint4* __restrict__ x, int V, int k, int E, const int32_t* __restrict__ idx,
-                    const int32_t* __restrict__ chunk_base, void* __restrict__ x_perm_v, float* __restrict__ xs,
+    dispatch_kernel(const uint4* x, int V, int k, int E, const int32_t* idx, const int32_t* chunk_base,
+                    void* __restrict__ x_perm_v, float* __restrict__ xs,
                     uint2* __restrict__ xq_sh, float* __restrict__ xs_sh, int32_t* __restrict__ perm_src,
                     int32_t* __restrict__ perm_dst, uint32_t* status, const DispatchSeg seg) {
   pdl_wait();
@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kDispatchThreads)
 }
 
 // The claimed post of a round that holds combined token tg.
-__device__ __forceinline__ int mbox_post(const MboxRound* __restrict__ r, int tg) {
+__device__ __forceinline__ int mbox_post(const MboxRound* r, int tg) {
   int lo = 0, hi = r->count;  // the last claimed post starting at or before tg
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
@@ -202,8 +202,8 @@ __device__ __forceinline__ int mbox_post(const MboxRound* __restrict__ r, int tg
 // region.
 template <bool FP8>
 __global__ void __launch_bounds__(kDispatchThreads)
-    dispatch_mbox_kernel(const MboxRound* __restrict__ r, const MboxGeom g, const int32_t* __restrict__ idx,
-                         const int32_t* __restrict__ chunk_base, const int32_t* __restrict__ offsets,
+    dispatch_mbox_kernel(const MboxRound* r, const MboxGeom g, const int32_t* idx, const int32_t* chunk_base,
+                         const int32_t* offsets,
                          void* __restrict__ x_perm_v, float* __restrict__ xs, void* __restrict__ x_sh,
                          float* __restrict__ xs_sh, int32_t* __restrict__ perm_src, int32_t* __restrict__ perm_dst,
                          uint32_t* status) {
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(kDispatchThreads)
 }
 
 // Rows of bf16 to e4m3 with a scale per 128 channels; one warp per row.
-__global__ void __launch_bounds__(256) quantize_rows_kernel(const uint4* __restrict__ x, int rows, int V,
+__global__ void __launch_bounds__(256) quantize_rows_kernel(const uint4* x, int rows, int V,
                                                             uint2* __restrict__ q, float* __restrict__ s) {
   pdl_wait();
   pdl_launch();
@@ -240,12 +240,47 @@ __global__ void __launch_bounds__(256) quantize_rows_kernel(const uint4* __restr
   const long long r = static_cast<long long>(blockIdx.x) * 8 + warp;
   if (r >= rows) return;
   const int nb = V / 16;
-  for (int v = lane; v < V; v += 32) {
-    float scale;
-    const uint2 w = quantize8(__ldg(x + r * V + v), scale);
-    q[r * V + v] = w;
-    if ((lane & 15) == 0) s[r * nb + (v >> 4)] = scale;
+  constexpr int kAhead = 4;  // vectors of the row per lane in flight
+  for (int v0 = lane; v0 < V; v0 += 32 * kAhead) {
+    uint4 a[kAhead];
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i)
+      if (v0 + 32 * i < V) a[i] = ld_dep(x + r * V + v0 + 32 * i);
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+      const int v = v0 + 32 * i;
+      if (v >= V) break;
+      float scale;
+      q[r * V + v] = quantize8(a[i], scale);
+      if ((lane & 15) == 0) s[r * nb + (v >> 4)] = scale;
+    }
   }
+}
+
+// acc += w y for a vector of eight bf16; the shared expert's row is added plainly.
+__device__ __forceinline__ void add_row(float (&acc)[8], float w, const uint4& y) {
+  acc[0] = fmaf(w, bf16_lo(y.x), acc[0]);
+  acc[1] = fmaf(w, bf16_hi(y.x), acc[1]);
+  acc[2] = fmaf(w, bf16_lo(y.y), acc[2]);
+  acc[3] = fmaf(w, bf16_hi(y.y), acc[3]);
+  acc[4] = fmaf(w, bf16_lo(y.z), acc[4]);
+  acc[5] = fmaf(w, bf16_hi(y.z), acc[5]);
+  acc[6] = fmaf(w, bf16_lo(y.w), acc[6]);
+  acc[7] = fmaf(w, bf16_hi(y.w), acc[7]);
+}
+__device__ __forceinline__ void add_shared(float (&acc)[8], const uint4& s) {
+  acc[0] += bf16_lo(s.x);
+  acc[1] += bf16_hi(s.x);
+  acc[2] += bf16_lo(s.y);
+  acc[3] += bf16_hi(s.y);
+  acc[4] += bf16_lo(s.z);
+  acc[5] += bf16_hi(s.z);
+  acc[6] += bf16_lo(s.w);
+  acc[7] += bf16_hi(s.w);
+}
+__device__ __forceinline__ uint4 pack_row(const float (&acc)[8]) {
+  return make_uint4(pack_bf16x2(acc[0], acc[1]), pack_bf16x2(acc[2], acc[3]), pack_bf16x2(acc[4], acc[5]),
+                    pack_bf16x2(acc[6], acc[7]));
 }
 
 constexpr int kCombineThreads = 256;
@@ -261,9 +296,8 @@ constexpr int kCombineCtas = 3;  // per SM (register cap)
 // 12 / 21 / 81 / 119 / 422.)
 // The body for one token: w_t, pd_t its k weights and positions, y_sh_t its
 // shared-expert row (nullable), out_t its output row.
-__device__ __forceinline__ void combine_token(const uint4* __restrict__ y_perm, const uint4* __restrict__ y_sh_t,
-                                              const float* __restrict__ w_t, const int32_t* __restrict__ pd_t, int V,
-                                              int k, uint4* __restrict__ out_t, uint32_t* status, long long nk) {
+__device__ __forceinline__ void combine_token(const uint4* y_perm, const uint4* y_sh_t, const float* w_t,
+                                              const int32_t* pd_t, int V, int k, uint4* __restrict__ out_t, uint32_t* status, long long nk) {
   int p[kMaxTopK];
   float wj[kMaxTopK];
 #pragma unroll
@@ -284,44 +318,21 @@ __device__ __forceinline__ void combine_token(const uint4* __restrict__ y_perm, 
     uint4 yv[kMaxTopK];
 #pragma unroll
     for (int j = 0; j < kMaxTopK; ++j)
-      if (p[j] >= 0) yv[j] = __ldg(y_perm + static_cast<long long>(p[j]) * V + v);
+      if (p[j] >= 0) yv[j] = ld_dep(y_perm + static_cast<long long>(p[j]) * V + v);
     float acc[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) acc[q] = 0.f;
 #pragma unroll
-    for (int j = 0; j < kMaxTopK; ++j) {
-      if (p[j] >= 0) {
-        const float a = wj[j];
-        acc[0] = fmaf(a, bf16_lo(yv[j].x), acc[0]);
-        acc[1] = fmaf(a, bf16_hi(yv[j].x), acc[1]);
-        acc[2] = fmaf(a, bf16_lo(yv[j].y), acc[2]);
-        acc[3] = fmaf(a, bf16_hi(yv[j].y), acc[3]);
-        acc[4] = fmaf(a, bf16_lo(yv[j].z), acc[4]);
-        acc[5] = fmaf(a, bf16_hi(yv[j].z), acc[5]);
-        acc[6] = fmaf(a, bf16_lo(yv[j].w), acc[6]);
-        acc[7] = fmaf(a, bf16_hi(yv[j].w), acc[7]);
-      }
-    }
-    if (y_sh_t) {
-      const uint4 s = __ldg(y_sh_t + v);
-      acc[0] += bf16_lo(s.x);
-      acc[1] += bf16_hi(s.x);
-      acc[2] += bf16_lo(s.y);
-      acc[3] += bf16_hi(s.y);
-      acc[4] += bf16_lo(s.z);
-      acc[5] += bf16_hi(s.z);
-      acc[6] += bf16_lo(s.w);
-      acc[7] += bf16_hi(s.w);
-    }
-    out_t[v] = make_uint4(pack_bf16x2(acc[0], acc[1]), pack_bf16x2(acc[2], acc[3]), pack_bf16x2(acc[4], acc[5]),
-                          pack_bf16x2(acc[6], acc[7]));
+    for (int j = 0; j < kMaxTopK; ++j)
+      if (p[j] >= 0) add_row(acc, wj[j], yv[j]);
+    if (y_sh_t) add_shared(acc, ld_dep(y_sh_t + v));
+    out_t[v] = pack_row(acc);
   }
 }
 
 __global__ void __launch_bounds__(kCombineThreads, kCombineCtas)
-    combine_kernel(const uint4* __restrict__ y_perm, const uint4* __restrict__ y_sh,
-                   const float* __restrict__ w, const int32_t* __restrict__ perm_dst, int V,
-                   int k, uint4* __restrict__ out, uint32_t* status, long long nk) {
+    combine_kernel(const uint4* y_perm, const uint4* y_sh, const float* w, const int32_t* perm_dst, int V, int k,
+                   uint4* __restrict__ out, uint32_t* status, long long nk) {
   pdl_wait();
   pdl_launch();
   const int t = blockIdx.x;
@@ -334,9 +345,8 @@ __global__ void __launch_bounds__(kCombineThreads, kCombineCtas)
 // token's post writes into its own output; its weights and positions are in its
 // slot's region, its shared-expert row at its place in the combined order.
 __global__ void __launch_bounds__(kCombineThreads, kCombineCtas)
-    combine_mbox_kernel(const MboxRound* __restrict__ r, const MboxGeom g, const uint4* __restrict__ y_perm,
-                        const uint4* __restrict__ y_sh, const float* __restrict__ w,
-                        const int32_t* __restrict__ perm_dst, uint32_t* status) {
+    combine_mbox_kernel(const MboxRound* r, const MboxGeom g, const uint4* y_perm, const uint4* y_sh, const float* w,
+                        const int32_t* perm_dst, uint32_t* status) {
   pdl_wait();
   pdl_launch();
   const int n_total = r->n_total;

@@ -29,7 +29,7 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kRouterEB = 16;    // experts per pass
 constexpr int kRouterAhead = 8;  // row pieces in flight per lane
 
-__global__ void __launch_bounds__(256) router_small_kernel(const uint4* __restrict__ x, LayerRef lref,
+__global__ void __launch_bounds__(256) router_small_kernel(const uint4* x, LayerRef lref,
                                                            uint32_t* status, int n, int V, int E,
                                                            float* __restrict__ logits) {
   pdl_wait();
@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(256) router_small_kernel(const uint4* __restri
 #pragma unroll
       for (int u = 0; u < kRouterAhead; ++u) {
         const int v = v0 + 32 * u;
-        xv[u] = v < V ? __ldg(xr + v) : make_uint4(0, 0, 0, 0);
+        xv[u] = v < V ? ld_dep(xr + v) : make_uint4(0, 0, 0, 0);
       }
 #pragma unroll
       for (int u = 0; u < kRouterAhead; ++u) {
@@ -112,7 +112,7 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], uint32_t a0, uint3
 }
 
 template <int NB>  // E = 8 NB experts
-__global__ void __launch_bounds__(kRmmaWarps * 32) router_mma_kernel(const uint4* __restrict__ x, LayerRef lref,
+__global__ void __launch_bounds__(kRmmaWarps * 32) router_mma_kernel(const uint4* x, LayerRef lref,
                                                                      uint32_t* status, int n, int V,
                                                                      float* __restrict__ logits) {
   pdl_wait();
@@ -135,8 +135,8 @@ __global__ void __launch_bounds__(kRmmaWarps * 32) router_mma_kernel(const uint4
   // chunk ch covers 16-byte vectors 4 ch .. 4 ch + 3 of every row
   for (int ch = warp; ch < V / 4; ch += kRmmaWarps) {
     const int v = 4 * ch + q;
-    const uint4 a = in0 ? __ldg(x0 + v) : zero;
-    const uint4 b = in1 ? __ldg(x1 + v) : zero;
+    const uint4 a = in0 ? ld_dep(x0 + v) : zero;
+    const uint4 b = in1 ? ld_dep(x1 + v) : zero;
 #pragma unroll
     for (int j = 0; j < NB; ++j) {
       const uint4 w = __ldg(wr + static_cast<long long>(8 * j + g) * V + v);
@@ -235,7 +235,7 @@ constexpr int kGateWarps = kChunkTokens;  // one warp per token of the chunk
 // added in slice order.  Lane l holds experts l, l+32, ..., so expert order
 // and (i, lane) order agree.  The chunk's expert histogram is written
 // chunk-major: hist[chunk * E + e].
-__global__ void __launch_bounds__(kGateWarps * 32) gate_kernel(const float* __restrict__ logits, int splits,
+__global__ void __launch_bounds__(kGateWarps * 32) gate_kernel(const float* logits, int splits,
                                                                long long plane, int n, GateParams p,
                                                                int32_t* __restrict__ idx,
                                                                float* __restrict__ wout,
@@ -445,7 +445,7 @@ __device__ __forceinline__ void team_argmax(float& v, int& i, float& x) {
 // SCAN: the launch is one cluster with every chunk of the call (CTAs past the
 // last chunk have no tokens) and also scans: chunk_base, counts, offsets.
 template <int T, int S, bool SCAN>
-__global__ void __launch_bounds__(kChunkTokens * T) gate_team_kernel(const float* __restrict__ logits, int splits,
+__global__ void __launch_bounds__(kChunkTokens * T) gate_team_kernel(const float* logits, int splits,
                                                                  long long plane, int n, GateParams p,
                                                                  int32_t* __restrict__ idx,
                                                                  float* __restrict__ wout,
@@ -476,7 +476,7 @@ __global__ void __launch_bounds__(kChunkTokens * T) gate_team_kernel(const float
     if constexpr (S % 4 == 0) {
 #pragma unroll
       for (int v = 0; v < S / 4; ++v) {
-        const float4 a = __ldg(reinterpret_cast<const float4*>(row) + v);
+        const float4 a = ld_dep(reinterpret_cast<const float4*>(row) + v);
         l[4 * v] = a.x;
         l[4 * v + 1] = a.y;
         l[4 * v + 2] = a.z;
@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(kChunkTokens * T) gate_team_kernel(const float
       for (int s2 = 1; s2 < splits; ++s2) {
 #pragma unroll
         for (int v = 0; v < S / 4; ++v) {
-          const float4 a = __ldg(reinterpret_cast<const float4*>(row + s2 * plane) + v);
+          const float4 a = ld_dep(reinterpret_cast<const float4*>(row + s2 * plane) + v);
           l[4 * v] += a.x;
           l[4 * v + 1] += a.y;
           l[4 * v + 2] += a.z;
@@ -496,8 +496,8 @@ __global__ void __launch_bounds__(kChunkTokens * T) gate_team_kernel(const float
     } else {
 #pragma unroll
       for (int j = 0; j < S; ++j) {
-        float a = __ldg(row + j);
-        for (int s2 = 1; s2 < splits; ++s2) a += __ldg(row + s2 * plane + j);
+        float a = ld_dep(row + j);
+        for (int s2 = 1; s2 < splits; ++s2) a += ld_dep(row + s2 * plane + j);
         l[j] = a;
       }
     }
@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(kChunkTokens * T) gate_team_kernel(const float
 }
 
 // ------------------------------------------------------------ histogram only
-__global__ void __launch_bounds__(256) hist_kernel(const int32_t* __restrict__ idx, int n, int k, int E,
+__global__ void __launch_bounds__(256) hist_kernel(const int32_t* idx, int n, int k, int E,
                                                    int32_t* __restrict__ hist, uint32_t* status) {
   pdl_wait();
   pdl_launch();
@@ -646,7 +646,7 @@ __global__ void __launch_bounds__(256) hist_kernel(const int32_t* __restrict__ i
 // launch: a cluster whose CTAs take consecutive chunk ranges.
 constexpr int kHistScanCtas = 8, kHistScanChunks = 32, kHistScanThreads = 1024;
 
-__global__ void __launch_bounds__(kHistScanThreads) hist_scan_kernel(const int32_t* __restrict__ idx, int n, int k,
+__global__ void __launch_bounds__(kHistScanThreads) hist_scan_kernel(const int32_t* idx, int n, int k,
                                                                      int E, int per, int32_t* __restrict__ counts,
                                                                      int32_t* __restrict__ offsets,
                                                                      int32_t* __restrict__ chunk_base,
@@ -662,8 +662,17 @@ __global__ void __launch_bounds__(kHistScanThreads) hist_scan_kernel(const int32
   const int ec = kChunkTokens * k;  // entries of a chunk
   const int32_t* mine = idx + static_cast<long long>(c0) * ec;
   const int ne = (min(n, c1 * kChunkTokens) - min(n, c0 * kChunkTokens)) * k;
-  for (int i = threadIdx.x; i < ne; i += kHistScanThreads) {
-    const int e = mine[i];
+  constexpr int kEach = kHistScanChunks * kChunkTokens * kMaxTopK / kHistScanThreads;  // entries per thread at most
+  int mine_e[kEach];
+#pragma unroll
+  for (int u = 0; u < kEach; ++u) {
+    const int i = threadIdx.x + u * kHistScanThreads;
+    mine_e[u] = i < ne ? ld_dep(mine + i) : 0;
+  }
+#pragma unroll
+  for (int u = 0; u < kEach; ++u) {
+    const int i = threadIdx.x + u * kHistScanThreads, e = mine_e[u];
+    if (i >= ne) break;
     if (e >= 0 && e < E) atomicAdd(&h[i / ec * E + e], 1);
     else record_status(status, ST_BAD_EXPERT_INDEX);
   }
@@ -706,15 +715,16 @@ constexpr int kScanAhead = 32;
 // of hist, in that order (n_chunks is then rowmap's length), and chunk_base
 // is written at the same rows.
 template <bool MAPPED>
-__global__ void __launch_bounds__(kScanWarps * 32) scan_kernel(const int32_t* __restrict__ hist, int n_chunks, int E,
+__global__ void __launch_bounds__(kScanWarps * 32) scan_kernel(const int32_t* hist, int n_chunks, int E,
                                                                int32_t* __restrict__ counts,
                                                                int32_t* __restrict__ offsets,
                                                                int32_t* __restrict__ chunk_base,
                                                                int32_t* __restrict__ tile_counters,
-                                                               const int32_t* __restrict__ rowmap,
-                                                               const int32_t* __restrict__ n_chunks_dev) {
+                                                               const int32_t* rowmap,
+                                                               const int32_t* n_chunks_dev) {
   __shared__ int part[kScanWarps][32];
   __shared__ int blk[kMaxExperts / 32];  // sums of the CTAs before this one
+  __shared__ int rows[MAPPED ? kScanWarps : 1][32];  // rowmap entries of each warp's batch of chunks
   // every CTA of the cluster has started: its shared memory may be written
   asm volatile("barrier.cluster.arrive.release;" ::: "memory");
   pdl_wait();
@@ -723,14 +733,23 @@ __global__ void __launch_bounds__(kScanWarps * 32) scan_kernel(const int32_t* __
   const int rank = blockIdx.x, ranks = gridDim.x;
   const int e = rank * 32 + lane;
   const bool ve = e < E;
-  if constexpr (MAPPED) n_chunks = max(0, min(*n_chunks_dev, n_chunks));  // n_chunks: rowmap's length
-  auto at = [&](int c) -> long long { return static_cast<long long>(MAPPED ? rowmap[c] : c) * E + e; };
+  if constexpr (MAPPED) n_chunks = max(0, min(ld_dep(n_chunks_dev), n_chunks));  // n_chunks: rowmap's length
   const int per = (n_chunks + kScanWarps - 1) / kScanWarps;
   const int c0 = min(n_chunks, g * per), c1 = min(n_chunks, c0 + per);
+  static_assert(kScanAhead == 32, "a lane reads the row of one chunk of the batch");
   int v[kScanAhead];
+  // (volatile: 32 rows kept in registers beside v would spill)
+  auto at = [&](int c, int u) -> long long {
+    return static_cast<long long>(MAPPED ? *static_cast<volatile int*>(&rows[g][u]) : c + u) * E + e;
+  };
   auto load = [&](int c) {
+    if constexpr (MAPPED) {
+      __syncwarp();
+      if (c + lane < c1) rows[g][lane] = ld_dep(rowmap + c + lane);
+      __syncwarp();
+    }
 #pragma unroll
-    for (int u = 0; u < kScanAhead; ++u) v[u] = ve && c + u < c1 ? hist[at(c + u)] : 0;
+    for (int u = 0; u < kScanAhead; ++u) v[u] = ve && c + u < c1 ? ld_dep(hist + at(c, u)) : 0;
   };
   int sum = 0;
   for (int c = c0; c < c1; c += kScanAhead) {
@@ -764,7 +783,7 @@ __global__ void __launch_bounds__(kScanWarps * 32) scan_kernel(const int32_t* __
     if (per > kScanAhead) load(c);
 #pragma unroll
     for (int u = 0; u < kScanAhead; ++u) {
-      if (ve && c + u < c1) chunk_base[at(c + u)] = run;
+      if (ve && c + u < c1) chunk_base[at(c, u)] = run;
       run += v[u];
     }
   }
@@ -781,14 +800,14 @@ __global__ void __launch_bounds__(kScanWarps * 32) scan_kernel(const int32_t* __
 }
 
 // Sum of the K-slice planes of the router GEMM, added in slice order.
-__global__ void reduce_splits_kernel(const float* __restrict__ parts, int splits, long long plane,
+__global__ void reduce_splits_kernel(const float* parts, int splits, long long plane,
                                      float* __restrict__ out) {
   pdl_wait();
   pdl_launch();
   for (long long i = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; i < plane;
        i += static_cast<long long>(gridDim.x) * blockDim.x) {
-    float v = parts[i];
-    for (int s2 = 1; s2 < splits; ++s2) v += parts[s2 * plane + i];
+    float v = ld_dep(parts + i);
+    for (int s2 = 1; s2 < splits; ++s2) v += ld_dep(parts + s2 * plane + i);
     out[i] = v;
   }
 }
