@@ -142,8 +142,7 @@ __device__ __forceinline__ bool produce(const GemmArgs& args, const MapsF8& maps
   while (ok) {
     ok = __all_sync(0xffffffffu, tq.pop(T, abort_flag));
     if (!ok) break;
-    if (issuer) tq.release();
-    ++tq.n;
+    tq.release(issuer);
     if (T.k_iters == 0) return true;
     // weights: box (w_tile, kb) is rows (w_tile k_iters + kb) 256 of 128
     // bytes; tokens: a box of the next multiple of 32 rows
@@ -273,8 +272,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       while (ok) {
         ok = __all_sync(0xffffffffu, tq.pop(T, abort_flag));
         if (!ok) break;
-        if (issuer) tq.release();
-        ++tq.n;
+        tq.release(issuer);
         if (T.k_iters == 0) break;
         for (int kb = 0; kb < T.k_iters; ++kb) {
           // the stages' operands and the partial, a third of the lanes each
@@ -341,8 +339,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     auto pop_next = [&]() -> bool {
       const bool got = __all_sync(0xffffffffu, tq.pop(next, abort_flag));
       if (!got) return false;
-      if (lane == 0) tq.release();
-      ++tq.n;
+      tq.release(lane == 0);
       const int valid = next.rows - q * 32;
       if (next.k_iters == 0 || valid <= 0) return true;
       const int sld = next.p1 ? fa.a_sld1 : fa.a_sld0;

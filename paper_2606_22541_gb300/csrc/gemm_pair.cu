@@ -16,7 +16,8 @@
 //   warp 1: TMEM; in the leader the MMA issuer of the pair
 //   warps 2-5: epilogue, one TMEM lane quarter each
 //   warp 6: token producer (its half of the tile's rows)
-//   warp 7: in the leader the tile scheduler of the pair
+//   warp 7: in the leader the tile scheduler of the pair, in the other CTA the
+//           thread that passes tile releases on to it
 // All loads complete on the leader's full barriers; the leader's commits
 // arrive on both CTAs' empty and accumulator barriers.
 //
@@ -50,8 +51,10 @@ constexpr int kNumBars = 2 * SW + 2 * SX + 5;
 constexpr int kBarBytes = (8 * kNumBars + 15) / 16 * 16 + kPairQBytes + 16;
 constexpr size_t kSmem = SW * kWBytes + SX * kXBytes + kStageBytes + kBarBytes + sizeof(MixSched);
 static_assert(kSmem <= 227 * 1024, "shared memory budget");
-// consumers of a tile: both CTAs' producers and epilogue warps, the MMA issuer
-constexpr int kQueueConsumers = 2 * (2 + kEpiWarps) + 1;
+// consumers of a tile: in each CTA the producers and the epilogue warps, in the
+// leader also the MMA issuer and the other CTA's forwarding thread
+constexpr int kQueueReaders = 2 + kEpiWarps;
+constexpr int kQueueConsumers = kQueueReaders + 2;
 
 struct PairMaps {
   CUtensorMap x[2][4];  // problem; boxes of 32, 64, 96 and 128 token rows
@@ -207,8 +210,7 @@ __device__ __forceinline__ bool produce(const GemmArgs& args, const PairMaps& ma
   PairTile T;
   while (true) {
     if (!__all_sync(0xffffffffu, tq.pop(T, abort_flag))) return false;
-    if (issuer) tq.release();
-    ++tq.n;
+    tq.release(issuer);
     if (T.k_iters == 0) break;
     // weights: box (w_tile, kb) is rows (w_tile k_iters + kb) 256 of 64
     // columns, this CTA loads its half of it; tokens: the CTA's half of the
@@ -291,6 +293,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       for (int s = 0; s < kPairQ; ++s) {
         mbar_init(PairQueue::full(tq0, s), 1);
         mbar_init(PairQueue::empty(tq0, s), kQueueConsumers);
+        mbar_init(PairQueue::read(tq0, s), kQueueReaders);
       }
       *abort_flag = 0;
       fence_barrier_init();
@@ -340,6 +343,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     // ------------------------------------------------------------ scheduler
     if (!pair_schedule<kPairRows>(args, sch, G, tq, pair_map(tq0, 1), abort_flag)) give_up();
     pdl_launch();  // no tiles left for this pair
+  } else if (warp == kSchedWarp && lane == 0) {
+    if (!pair_forward(tq, abort_flag)) give_up();
   } else if (warp == 1 && leader) {
     // ------------------------------------------------------------ MMA issuer
     // the whole warp runs the loop, one lane issues
@@ -353,8 +358,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     for (int it = 0; ok; ++it) {
       ok = __all_sync(0xffffffffu, tq.pop(T, abort_flag));
       if (!ok) break;
-      if (issuer) tq.release();
-      ++tq.n;
+      tq.release(issuer);
       if (T.k_iters == 0) break;
       const int acc = it & 1;
       ok = __all_sync(0xffffffffu, mbar_wait(tempty(acc), ((it >> 1) & 1) ^ 1u, abort_flag));
@@ -403,11 +407,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     PairTile T;
     for (int it = 0;; ++it) {
       const int acc = it & 1;
-      bool ok = tq.pop(T, abort_flag);
-      __syncwarp();
+      bool ok = __all_sync(0xffffffffu, tq.pop(T, abort_flag));
       if (ok) {
-        if (lane == 0) tq.release();
-        ++tq.n;
+        tq.release(lane == 0);
         if (T.k_iters > 0) ok = mbar_wait(tfull(acc), (it >> 1) & 1, abort_flag);
       }
       // the four warps share barriers below: all go on or none does

@@ -41,12 +41,33 @@ __device__ __forceinline__ void st_pair_u32(uint32_t addr, uint32_t v) {
   asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 // Arrive on a barrier of either CTA (addr from pair_map).  Without .cluster
-// scope here and in the waits: what these barriers order is TMEM (fenced by
-// tcgen05) and registers; a cluster-scope release or acquire stalled its thread
-// for 2000 to 4000 cycles behind the loads in flight (tile changes took 300
-// cycles without it; gate/up GEMM of 8192 DeepSeek-V3 tokens 3059 -> 2917 us).
+// scope: what it orders is TMEM (fenced by tcgen05); a cluster-scope release or
+// acquire stalled its thread for 2000 to 4000 cycles behind the loads in flight
+// (tile changes took 300 cycles without it; gate/up GEMM of 8192 DeepSeek-V3
+// tokens 3059 -> 2917 us).
 __device__ __forceinline__ void mbar_arrive_pair(uint32_t addr) {
   asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+// The same with cluster scope, and the wait for it: this CTA's reads of its
+// shared memory, its own and those it has waited for, come before what the
+// waiting thread of the other CTA does next.
+__device__ __forceinline__ void mbar_arrive_release_pair(uint32_t addr) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+__device__ __forceinline__ bool mbar_wait_acquire_pair(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return bounded_wait(
+      [&]() {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        return ok != 0;
+      },
+      abort_flag);
 }
 // Arrive on the other CTA's barrier and expect ``bytes`` of st.async on it.
 __device__ __forceinline__ void mbar_arrive_expect_tx_pair(uint32_t addr, uint32_t bytes) {
@@ -236,15 +257,18 @@ __device__ __forceinline__ void pair_decode(int t, const MixSched* s, int G, int
 // ---------------------------------------------------------------- tile queue
 // One CTA of the pair is the queue's home: its scheduler thread claims tiles,
 // decodes them and writes the descriptions into both CTAs' queues, one tile
-// ahead of the loads; the consumers of both CTAs release a slot on the home's
-// barrier.  (With every
-// role popping an id and decoding it itself, the id claimed when the loads
+// ahead of the loads.  The consumers release a slot on a barrier of their own
+// CTA: the home's on the empty barrier, the other CTA's on its read barrier,
+// whose completions a thread without loads of its own (pair_forward) passes on
+// to the home with cluster scope, so that the other CTA's reads of a slot come
+// before the home's next store into it and no role pays for the scope.  (With
+// every role popping an id and decoding it itself, the id claimed when the loads
 // reached it, a tile change cost the MMA issuer about 3200 cycles.)
 constexpr int kPairQ = 2;
-constexpr int kPairQBytes = kPairQ * (static_cast<int>(sizeof(PairTile)) + 16);
+constexpr int kPairQBytes = kPairQ * (static_cast<int>(sizeof(PairTile)) + 24);
 
 struct PairQueue {
-  uint32_t q0;    // this CTA's queue: descriptions, full and empty barriers
+  uint32_t q0;    // this CTA's queue: descriptions, full, empty and read barriers
   uint32_t home;  // the home's, in the cluster window
   bool at_home;   // this CTA is the home
   uint32_t n = 0;
@@ -254,6 +278,7 @@ struct PairQueue {
   __device__ __forceinline__ static uint32_t desc(uint32_t b, uint32_t s) { return b + 32u * s; }
   __device__ __forceinline__ static uint32_t full(uint32_t b, uint32_t s) { return b + 32u * kPairQ + 8u * s; }
   __device__ __forceinline__ static uint32_t empty(uint32_t b, uint32_t s) { return b + 40u * kPairQ + 8u * s; }
+  __device__ __forceinline__ static uint32_t read(uint32_t b, uint32_t s) { return b + 48u * kPairQ + 8u * s; }
 
   __device__ __forceinline__ static void store_local(uint32_t addr, const PairTile& T) {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(T.row), "r"(T.rows), "r"(T.n),
@@ -266,7 +291,7 @@ struct PairQueue {
   // scheduler thread; peer: the other CTA's queue in the cluster window
   __device__ __forceinline__ bool push(const PairTile& T, uint32_t peer, volatile int* abort_flag) {
     const uint32_t s = slot();
-    if (!mbar_wait(empty(q0, s), phase() ^ 1u, abort_flag)) return false;
+    if (!mbar_wait_acquire_pair(empty(q0, s), phase() ^ 1u, abort_flag)) return false;
     const uint32_t pd = desc(peer, s), pb = full(peer, s), ld = desc(q0, s);
     mbar_arrive_expect_tx_pair(pb, 32);
     st_async_v4(pd, pb, T.row, T.rows, T.n, T.w_tile);
@@ -276,7 +301,7 @@ struct PairQueue {
     ++n;
     return true;
   }
-  // any number of threads of a role; the role releases the slot once
+  // whole warps; a role's warp releases the slot once
   __device__ __forceinline__ bool pop(PairTile& T, volatile int* abort_flag) const {
     const uint32_t s = slot();
     if (!mbar_wait(full(q0, s), phase(), abort_flag)) return false;
@@ -291,11 +316,28 @@ struct PairQueue {
                  : "memory");
     return true;
   }
-  __device__ __forceinline__ void release() const {
-    if (at_home) mbar_arrive(empty(q0, slot()));
-    else mbar_arrive_pair(empty(home, slot()));
+  // the whole warp calls this once every lane has popped; one lane arrives and
+  // the warp goes on to the next slot
+  __device__ __forceinline__ void release(bool one) {
+    __syncwarp();  // the other lanes' reads come before the arrival
+    if (one) mbar_arrive(at_home ? empty(q0, slot()) : read(q0, slot()));
+    ++n;
   }
 };
+
+// One thread of the CTA that is not the home: passes the releases of its CTA's
+// roles on to the home, until the end of the tiles.
+__device__ __forceinline__ bool pair_forward(PairQueue& tq, volatile int* abort_flag) {
+  PairTile T;
+  while (true) {
+    if (!tq.pop(T, abort_flag)) return false;
+    if (T.k_iters == 0) return true;
+    const uint32_t s = tq.slot();
+    if (!mbar_wait(PairQueue::read(tq.q0, s), tq.phase(), abort_flag)) return false;
+    mbar_arrive_release_pair(PairQueue::empty(tq.home, s));
+    ++tq.n;
+  }
+}
 
 // The same queue within one CTA (home and only consumer).
 __device__ __forceinline__ bool local_push(PairQueue& tq, const PairTile& T, volatile int* abort_flag) {
