@@ -188,7 +188,8 @@ int asap_moe_n_layers(asap_moe_t h, int32_t* n_layers);
  *  - ASAP_TILING_AUTO (the default): per launch, CTA pairs when the routed
  *    rows average at least 64 per expert or the launch has at most two waves
  *    of single-CTA tiles (from n, top_k and the expert count), else single
- *    CTAs.
+ *    CTAs; contractions below 1024 take pairs, single CTAs or single CTAs with
+ *    two 128-row m-tiles per tile by their length and the launch's size.
  *  - ASAP_TILING_SINGLE: one CTA per tile, tiles of 128 rows.
  *  - ASAP_TILING_PAIRED: two CTAs on the SMs of one TPC per tile, tiles of up
  *    to 256 rows of one expert (equal heights within a segment, in steps of

@@ -301,15 +301,13 @@ int run_route(asap_moe_t h, const void* x, int n, int32_t* idx, float* w, int32_
   return run_gate_scan(h, logits, splits, n, idx, w, counts, offsets, ws, layer, st);
 }
 
-// Paired m-tiles of the down GEMM with the fused combine (two 128-row m-tiles
-// per GEMM tile sharing the weight boxes, a half tile for a segment's last
-// <= 128 rows) when
+// Paired m-tiles of the single-CTA kernel (two 128-row m-tiles per GEMM tile
+// sharing the weight boxes, a half tile for a segment's last <= 128 rows), for
+// short contractions and the fused combine, when
 //  - the segments hold at least one m-tile (128 rows) per expert on average:
 //    below that nearly every paired tile is a half tile, and the paired rings
 //    (3 + 3 stages) keep fewer weight bytes in flight than the single-tile
-//    rings (4 + 4).  Measured on a GB300 at the DeepSeek-V3 shape (gate/up |
-//    down ms, paired vs single): 3072 tokens (96 rows per expert) 2.26 |
-//    1.23 vs 2.19 | 1.16; 4096 tokens (128) 2.35 | 1.31 vs 2.39 | 1.33;
+//    rings (4 + 4);
 //  - and the launch has at least ASAP_PAIR_MIN_WAVES waves of paired tiles
 //    (estimate: nk / 256 full tiles plus half a tile of rounding per
 //    non-empty segment).  With few tiles the larger tile rounds the launch to
@@ -338,17 +336,21 @@ int block_tiles(int rows, long long row_bytes) {
   return static_cast<int>(std::max<long long>(1, ASAP_BLOCK_BYTES / (rows * std::max<long long>(row_bytes, 1))));
 }
 
+// Tiles of a bf16 expert GEMM: one CTA and 128 rows, one CTA and two 128-row
+// m-tiles, or a CTA pair (gemm_pair.cu).
+enum class Tiles { kSingle, kTwoM, kCtaPair };
+
 // Launch of a bf16 expert GEMM: A operands in0 [nk, K0] and in1 [n, K1] (the
 // shared expert's, when a.m1 > 0), outputs a.out0 and a.out1.
-int launch_expert_gemm(asap_moe_t h, int epi, bool cta2, bool pair, const void* in0, long long nk, int K0,
-                       const void* in1, int n, int K1, asap::GemmArgs& a, cudaStream_t st) {
+int launch_expert_gemm(asap_moe_t h, int epi, Tiles kind, const void* in0, long long nk, int K0, const void* in1,
+                       int n, int K1, asap::GemmArgs& a, cudaStream_t st) {
   const bool sh = a.m1 > 0;
   std::string err;
   bool ok = true;
   auto enc = [&](CUtensorMap* m, const void* p, long long rows, long long cols, uint32_t box) {
     ok = ok && asap::encode_tmap_bf16(m, p, rows, cols, box, &err);
   };
-  if (cta2) {
+  if (kind == Tiles::kCtaPair) {
     CUtensorMap maps[10];
     for (int i = 0; i < 4; ++i) {
       enc(&maps[i], in0, nk, K0, 32 * (i + 1));
@@ -380,6 +382,7 @@ int launch_expert_gemm(asap_moe_t h, int epi, bool cta2, bool pair, const void* 
     maps[3] = maps[2];
   }
   if (!ok) return fail(ASAP_ERR_INVALID, "expert GEMM operand: " + err);
+  const bool pair = kind == Tiles::kTwoM;
   const int bm = pair ? 2 * asap::kGemmBM : asap::kGemmBM;
   const long long tiles = static_cast<long long>(ub_mtiles(h->cfg, nk, bm)) * a.n_tiles0 +
                           (sh ? static_cast<long long>(asap::ceil_div(n, bm)) * a.n_tiles1 : 0);
@@ -388,8 +391,8 @@ int launch_expert_gemm(asap_moe_t h, int epi, bool cta2, bool pair, const void* 
   return ASAP_OK;
 }
 
-// CTA pairs (gemm_pair.cu) when the segments hold at least 64 rows per expert
-// on average, or when the launch has at most two waves of single-CTA tiles.
+// CTA pairs when the segments hold at least 64 rows per expert on average, or
+// when the launch has at most two waves of single-CTA tiles.
 // Measured on a GB300 (gate/up | down us, pairs vs single CTAs):
 //  - DeepSeek-V3, balanced: 8192 tokens 3059 | 1692 vs 3590 | 1915, 4096
 //    tokens (128 rows per expert) 2327 | 1238 vs 2416 | 1282; below the line
@@ -399,15 +402,30 @@ int launch_expert_gemm(asap_moe_t h, int epi, bool cta2, bool pair, const void* 
 //    268 | 144 vs 265 | 141;
 //  - DeepSeek-V3, 1 token (9 experts, 144 gate/up tiles): 86 | 53 vs 109 | 65,
 //    two half-length waves of pairs instead of one wave of single CTAs.
-// Short contractions stay on single CTAs: a pair's set-up costs about 1 us more
-// (the tiny layer, K = 256 and 128: 41.6 vs 39.7 us for the whole layer).
-bool use_cta2(asap_moe_t h, long long nk, int n_tiles0, long long m1, int n_tiles1, int k_iters) {
-  if (h->tiling != ASAP_TILING_AUTO) return h->tiling == ASAP_TILING_PAIRED;
-  if (k_iters < 16) return false;
-  if (nk >= 64ll * h->cfg.n_experts) return true;
-  const long long tiles = std::min<long long>(h->cfg.n_experts, nk) * n_tiles0 +
-                          static_cast<long long>(asap::ceil_div(m1, asap::kGemmBM)) * n_tiles1;
-  return tiles <= 2ll * h->num_sms;
+// Contractions below 1024: a pair's set-up costs about 1 us more (the tiny
+// layer, K = 256 and 128: 41.6 vs 39.7 us for the whole layer) and its output
+// leaves through two SMs' narrower stores, so a pair needs more than one wave of
+// tiles and K >= 512 (gate/up) or 640 (down); below that, two m-tiles per CTA
+// from their own threshold on.  Single / two m-tiles / pairs, 64 experts of 512
+// rows: down to 7168 channels K = 128 117 / 101 / 194, 256 146 / 136 / 197, 384
+// 197 / 173 / 201, 512 237 / 211 / 208 (of 2048 rows 818 / 674 / 738), 640 281 /
+// 244 / 222, 768 320 / 281 / 242; gate/up to 4096 K = 256 177 / 175 / 203 (of 128
+// rows 68 / 77 / 72, of 2048 619 / 580 / 689), 512 266 / 253 / 218, 768 357 / 332 /
+// 264.
+Tiles pick_tiles(asap_moe_t h, bool down, long long nk, int n_tiles0, long long m1, int n_tiles1, int k_iters) {
+  if (h->tiling != ASAP_TILING_AUTO) return h->tiling == ASAP_TILING_PAIRED ? Tiles::kCtaPair : Tiles::kSingle;
+  const long long E = h->cfg.n_experts;
+  const long long m1_tiles = asap::ceil_div(m1, asap::kGemmBM) * static_cast<long long>(n_tiles1);
+  if (k_iters >= 16) {
+    const long long tiles = std::min<long long>(E, nk) * n_tiles0 + m1_tiles;
+    return nk >= 64 * E || tiles <= 2ll * h->num_sms ? Tiles::kCtaPair : Tiles::kSingle;
+  }
+  if (k_iters >= (down ? 10 : 8)) {
+    const long long tiles = static_cast<long long>(ub_mtiles(h->cfg, nk)) * n_tiles0 + m1_tiles;
+    return nk >= 64 * E && tiles > h->num_sms ? Tiles::kCtaPair : Tiles::kSingle;
+  }
+  if (!down && nk < 1024 * E) return Tiles::kSingle;
+  return use_pair(h, nk, n_tiles0, m1, n_tiles1) ? Tiles::kTwoM : Tiles::kSingle;
 }
 
 // GEMM1: h = silu(X Wg^T) * (X Wu^T) on the routed segments, plus the shared
@@ -445,8 +463,8 @@ int run_gate_up(asap_moe_t h, const void* x_perm, const int32_t* offsets, const 
   a.k_splits = 1;
   a.tile_counter = counter;
   a.b_tiled = 1;  // weights in tile-contiguous order (pack_layer)
-  const bool cta2 = use_cta2(h, nk, a.n_tiles0, a.m1, a.n_tiles1, a.k_iters0);
-  return launch_expert_gemm(h, asap::EPI_SWIGLU, cta2, false, x_perm, nk, c.hidden, x, n, c.hidden, a, st);
+  return launch_expert_gemm(h, asap::EPI_SWIGLU, pick_tiles(h, false, nk, a.n_tiles0, a.m1, a.n_tiles1, a.k_iters0),
+                            x_perm, nk, c.hidden, x, n, c.hidden, a, st);
 }
 
 // GEMM2: y = h Wd^T on the routed segments, plus the shared expert.
@@ -499,9 +517,10 @@ int run_down(asap_moe_t h, const void* hbuf, const int32_t* offsets, const void*
   a.comb_n = n;
   a.comb_k = c.top_k;
   // the fused combine runs in the single-CTA kernel's epilogue
-  const bool pair = use_pair(h, nk, a.n_tiles0, a.m1, a.n_tiles1);
-  const bool cta2 = !cf.cnt && use_cta2(h, nk, a.n_tiles0, a.m1, a.n_tiles1, a.k_iters0);
-  return launch_expert_gemm(h, asap::EPI_BF16, cta2, cf.cnt && pair, hbuf, nk, c.inter, hsh, n, c.shared_inter, a, st);
+  const Tiles kind = !cf.cnt ? pick_tiles(h, true, nk, a.n_tiles0, a.m1, a.n_tiles1, a.k_iters0)
+                     : use_pair(h, nk, a.n_tiles0, a.m1, a.n_tiles1) ? Tiles::kTwoM
+                                                                     : Tiles::kSingle;
+  return launch_expert_gemm(h, asap::EPI_BF16, kind, hbuf, nk, c.inter, hsh, n, c.shared_inter, a, st);
 }
 
 // counters: kTileCounters zeroed ints (or nullptr)

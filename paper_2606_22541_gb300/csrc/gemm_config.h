@@ -23,8 +23,8 @@
 #ifndef ASAP_RING_DN_B
 #define ASAP_RING_DN_B 4
 #endif
-// paired m-tiles (two 128-row m-tiles per tile sharing the weight boxes; the
-// down GEMM with the fused combine): A stages of 2 x 128 rows (32 KB) and B
+// paired m-tiles (two 128-row m-tiles per tile sharing the weight boxes; short
+// contractions and the down GEMM with the fused combine): A stages of 2 x 128 rows (32 KB) and B
 // boxes of 32 KB, 3 + 3 stages.
 #ifndef ASAP_RING_PAIR_A
 #define ASAP_RING_PAIR_A 3
@@ -32,9 +32,9 @@
 #ifndef ASAP_RING_PAIR_B
 #define ASAP_RING_PAIR_B 3
 #endif
-// The down GEMM with the fused combine runs paired m-tiles when it has at least
-// this many waves of them (estimated, one tile per SM per wave): with fewer
-// the larger tile rounds the launch to whole waves more coarsely than it saves.
+// A launch of those kinds runs paired m-tiles when it has at least this many
+// waves of them (estimated, one tile per SM per wave): with fewer the larger tile
+// rounds the launch to whole waves more coarsely than it saves.
 #ifndef ASAP_PAIR_MIN_WAVES
 #define ASAP_PAIR_MIN_WAVES 3
 #endif

@@ -8,8 +8,8 @@
 // the per-expert counts back (the bubble-free principle of Section 3.4.2).
 //
 // This is the single-CTA form: the router's logits, launches with few rows per
-// expert (bound by the weight stream) and the fused combine; the other expert
-// launches run on CTA pairs (gemm_pair.cu).
+// expert (bound by the weight stream), short contractions and the fused combine;
+// the other expert launches run on CTA pairs (gemm_pair.cu).
 //
 // Design (one CTA per SM, persistent, warp-specialised; 224 threads, 352 with
 // paired m-tiles):
@@ -673,7 +673,9 @@ static_assert(sizeof(Sched) + 0 <= 8192, "schedule table");
 
 cudaError_t gemm_set_attributes() {
   cudaError_t e = set_attr<EPI_SWIGLU, false>();
+  if (e == cudaSuccess) e = set_attr<EPI_SWIGLU, true>();
   if (e == cudaSuccess) e = set_attr<EPI_BF16, false>();
+  if (e == cudaSuccess) e = set_attr<EPI_BF16, true>();
   if (e == cudaSuccess) e = set_attr<EPI_BF16, false, true>();
   if (e == cudaSuccess) e = set_attr<EPI_BF16, true, true>();
   if (e == cudaSuccess) e = set_attr<EPI_F32, false>();
@@ -683,12 +685,11 @@ cudaError_t gemm_set_attributes() {
 cudaError_t gemm_launch(int epi, bool pair, const CUtensorMap* maps, const GemmArgs& args, int grid,
                         cudaStream_t stream) {
   if (grid <= 0) return cudaSuccess;
-  // paired m-tiles: the down GEMM with the fused combine only (gemm_pair.cu
-  // runs the other launches of that size)
-  if (pair && !(epi == EPI_BF16 && args.comb_cnt)) return cudaErrorInvalidValue;
-  if (epi == EPI_SWIGLU) return launch<EPI_SWIGLU, false>(maps, args, grid, stream);
-  if (epi != EPI_BF16) return launch<EPI_F32, false>(maps, args, grid, stream);
-  if (!args.comb_cnt) return launch<EPI_BF16, false>(maps, args, grid, stream);
+  if (epi == EPI_F32) return pair ? cudaErrorInvalidValue : launch<EPI_F32, false>(maps, args, grid, stream);
+  if (epi == EPI_SWIGLU)
+    return pair ? launch<EPI_SWIGLU, true>(maps, args, grid, stream) : launch<EPI_SWIGLU, false>(maps, args, grid, stream);
+  if (!args.comb_cnt)
+    return pair ? launch<EPI_BF16, true>(maps, args, grid, stream) : launch<EPI_BF16, false>(maps, args, grid, stream);
   return pair ? launch<EPI_BF16, true, true>(maps, args, grid, stream)
               : launch<EPI_BF16, false, true>(maps, args, grid, stream);
 }
