@@ -251,7 +251,9 @@ int asap_moe_router_logits(asap_moe_t h, const void* x, int32_t n, float* logits
  * deterministic.  For E = 256 with grouped sigmoid gating (1, 2, 4 or 8
  * groups) this is two kernel launches (router GEMM over a thread-block cluster
  * with gating and histogram, then the scan); the logits are not written.
- * Other configurations launch the router, gate and scan kernels in turn. */
+ * Other configurations launch the router, gate and scan kernels in turn; up to
+ * 256 tokens the common expert counts (8, 16, 32, 64, 128, 256) scan in the gate's
+ * launch. */
 int asap_moe_route(asap_moe_t h, const void* x, int32_t n, int32_t* idx, float* w,
                    int32_t* counts, int32_t* offsets, void* ws, size_t ws_bytes,
                    void* stream);

@@ -20,7 +20,7 @@
 struct LayerWeights {
   void* router_w = nullptr;      // [E, H] bf16
   float* router_bias = nullptr;  // [E] fp32 or nullptr
-  void* gate_up = nullptr;       // [E][2I, H], gate/up interleaved per 128 rows
+  void* gate_up = nullptr;       // [E][2I, H], gate/up alternating in eights (bf16) or per 128 rows
   void* down = nullptr;          // [E][H, I]
   void* sh_gate_up = nullptr;    // [2Is, H]
   void* sh_down = nullptr;       // [H, Is]
@@ -814,8 +814,7 @@ int encode_layer(asap_moe_t h, const LayerWeights& L, asap::LayerEntry* out) {
     const uint64_t rows128 = rows * cols * wb / 128;
     CUtensorMap* m = &out->map[which];
     CUtensorMap* mp = &out->map[asap::MAP_PAIR + which];
-    return h->fp8 ? asap::encode_tmap_u8(m, p, rows128, 128, asap::kGemmBN, &err) &&
-                        asap::encode_tmap_u8(mp, p, rows128, 128, asap::kGemmBN / 2, &err)
+    return h->fp8 ? asap::encode_tmap_u8(m, p, rows128, 128, asap::kGemmBN, &err)
                   : asap::encode_tmap_bf16(m, p, rows128, 64, asap::kGemmBN, &err) &&
                         asap::encode_tmap_bf16(mp, p, rows128, 64, asap::kGemmBN / 2, &err);
   };
@@ -1211,7 +1210,7 @@ int run_layer_batched(asap_moe_t h, int32_t count, const void* const* xs, const 
       if ((r = run_router_logits(h, xs[i], n, lg, splits, layer, st)) != ASAP_OK) return r;
       CU_TRY(asap::launch_gate_seg(lg, splits, n, gate_params(h, layer),
                                    idx + static_cast<long long>(tok0) * k,
-                                   w + static_cast<long long>(tok0) * k, hist, chunk0, chunks_total, st),
+                                   w + static_cast<long long>(tok0) * k, hist, chunk0, st),
              "gate launch");
     }
     tok0 += n;
@@ -1231,7 +1230,6 @@ int run_layer_batched(asap_moe_t h, int32_t count, const void* const* xs, const 
       asap::DispatchSeg seg{};
       seg.expert_offsets = offsets;
       seg.chunk0 = chunk0;
-      seg.n_chunks_total = chunks_total;
       seg.tok0 = tok0;
       seg.rows_total = nk;
       const int32_t* idx_i = idx + static_cast<long long>(tok0) * k;
@@ -1533,7 +1531,7 @@ ASAP_API int asap_moe_mailbox_post(asap_moe_mailbox_t m, int32_t slot, const voi
   int32_t* idx = at<int32_t>(m->ws, m->L.idx) + sk;
   float* w = at<float>(m->ws, m->L.w) + sk;
   int32_t* hist = at<int32_t>(m->ws, m->L.hist);
-  const int chunk0 = slot * g.slot_chunks, chunks_total = g.n_slots * g.slot_chunks;
+  const int chunk0 = slot * g.slot_chunks;
   int r;
   if (n > 0) {
     // routing exactly as asap_moe_route routes n tokens; the histogram rows
@@ -1547,8 +1545,7 @@ ASAP_API int asap_moe_mailbox_post(asap_moe_mailbox_t m, int32_t slot, const voi
       float* lg = at<float>(m->ws, m->L.logits) +
                   static_cast<long long>(slot) * asap::kMaxRouterSplits * g.slot_tokens * c.n_experts;
       if ((r = run_router_logits(h, x, n, lg, splits, layer, st)) != ASAP_OK) return r;
-      CU_TRY(asap::launch_gate_seg(lg, splits, n, gate_params(h, layer), idx, w, hist, chunk0,
-                                   chunks_total, st),
+      CU_TRY(asap::launch_gate_seg(lg, splits, n, gate_params(h, layer), idx, w, hist, chunk0, st),
              "gate launch");
     }
   }

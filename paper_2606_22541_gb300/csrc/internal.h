@@ -50,7 +50,7 @@ enum { EPI_SWIGLU = 0, EPI_BF16 = 1, EPI_F32 = 2 };
 // the kernel loads from device memory when it runs.  The entry holds the TMA
 // descriptors of that layer's packed weights (the pre-computed addresses) and
 // plain pointers for what is not read by TMA.
-// (MAP_PAIR + MAP_*: the expert matrices again, for boxes of 128 rows.)
+// (MAP_PAIR + MAP_*: the bf16 expert matrices again, for boxes of 128 rows.)
 enum { MAP_ROUTER = 0, MAP_GATE_UP = 1, MAP_DOWN = 2, MAP_SH_GATE_UP = 3, MAP_SH_DOWN = 4, kLayerMats = 5,
        MAP_PAIR = 4, kLayerMaps = 9 };
 
@@ -110,8 +110,8 @@ constexpr int kGemmBN = 256;
 constexpr int kGemmBK = 64;
 
 cudaError_t gemm_set_attributes();
-// maps: A0, A1 (A1 may repeat A0 when m1 == 0), encoded for boxes of 128 rows,
-// or 256 rows with pair; then O0, O1, the bf16 outputs out0 / out1 encoded for
+// maps: A0, A1 (A1 may repeat A0 when m1 == 0), encoded for boxes of 128 rows;
+// then O0, O1, the bf16 outputs out0 / out1 encoded for
 // boxes of 32 rows (O1 may repeat O0 when m1 == 0; EPI_F32 ignores both).  The
 // B maps come from the layer table.  pair: tiles of two 128-row m-tiles
 // sharing the weight boxes (EPI_SWIGLU and EPI_BF16).
@@ -180,10 +180,9 @@ cudaError_t launch_gate(const float* logits, int splits, int n, const GateParams
                         int32_t* hist, cudaStream_t s);
 cudaError_t launch_reduce_splits(const float* parts, int splits, long long plane, float* out, cudaStream_t s);
 // Gating of one micro-batch among several served together: its chunks are
-// rows [chunk0, chunk0 + ceil(n/32)) of the chunk-major histogram with
-// n_chunks_total rows.
+// rows [chunk0, chunk0 + ceil(n/32)) of the chunk-major histogram.
 cudaError_t launch_gate_seg(const float* logits, int splits, int n, const GateParams& p, int32_t* idx, float* w,
-                            int32_t* hist, int chunk0, int n_chunks_total, cudaStream_t s);
+                            int32_t* hist, int chunk0, cudaStream_t s);
 // launch_gate and launch_scan of its histogram (hist: scratch that a call of few
 // chunks does not write).
 cudaError_t launch_gate_scan(const float* logits, int splits, int n, const GateParams& p, int32_t* idx, float* w,
@@ -227,14 +226,13 @@ cudaError_t launch_route_fused(const CUtensorMap& tmX, const RouteFusedArgs& a, 
 
 // ------------------------------------------------------------ permute
 // Place of one micro-batch among several served by one call: its chunks start
-// at column chunk0 of chunk_base (n_chunks_total columns), its tokens at
+// at row chunk0 of chunk_base, its tokens at
 // global index tok0, positions run over rows_total rows; x_sh (bf16 only,
 // nullable) receives its rows for the shared expert (pointer already offset
 // to the micro-batch's first token).
 struct DispatchSeg {
   const int32_t* expert_offsets;  // offsets[e] (the scan's output)
   int chunk0;
-  int n_chunks_total;
   int tok0;
   long long rows_total;
   void* x_sh;

@@ -80,11 +80,6 @@ __device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t bar, int a, 
                "r"(bar), "r"(a), "r"(b), "r"(c), "r"(d)
                : "memory");
 }
-__device__ __forceinline__ void st_async_v2(uint32_t addr, uint32_t bar, uint32_t a, uint32_t b) {
-  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%2, %3}, [%1];" ::"r"(addr),
-               "r"(bar), "r"(a), "r"(b)
-               : "memory");
-}
 // After a failed wait: copies this thread issued complete on a barrier of the
 // other CTA, which it cannot wait on, so it lets 2 ms pass (a TMA load takes
 // microseconds) before the CTA may wind down.
@@ -132,7 +127,7 @@ __device__ __forceinline__ void tc_mma_bf16_pair(uint32_t d_tmem, uint64_t adesc
 }
 
 // ---------------------------------------------------------------- fragments
-// 16 TMEM lanes x 64 (32, 16) columns.  Thread t receives, for each group n of 8
+// 16 TMEM lanes x 64 (32) columns.  Thread t receives, for each group n of 8
 // columns, lane t / 4 at columns 8n + 2 (t % 4), + 1 in r[4n], r[4n + 1] and
 // lane t / 4 + 8 at the same columns in r[4n + 2], r[4n + 3].
 __device__ __forceinline__ void tmem_ld_frag64(uint32_t taddr, uint32_t (&r)[32]) {
@@ -154,13 +149,6 @@ __device__ __forceinline__ void tmem_ld_frag32(uint32_t taddr, uint32_t (&r)[16]
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
         "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
         "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_ld_frag16(uint32_t taddr, uint32_t (&r)[16]) {  // r[0 .. 7]
-  asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
       : "r"(taddr)
       : "memory");
 }
@@ -206,8 +194,9 @@ __device__ __forceinline__ int mix_position(int t, int cold, int total) {
   constexpr int Q = ASAP_MIX_BURST;
   const int k = static_cast<int>(static_cast<long long>(t) * hot / (static_cast<long long>(Q) * total));
   const int tk = static_cast<int>((static_cast<long long>(k) * Q * total + hot - 1) / hot);
-  if (t >= tk && t - tk < Q && k * Q + t - tk < hot) return cold + k * Q + t - tk;
-  return t - min(t >= tk ? (k + 1) * Q : k * Q, hot);
+  // (t >= tk: k is the last burst that starts at or before t)
+  if (t - tk < Q && k * Q + t - tk < hot) return cold + k * Q + t - tk;
+  return t - min((k + 1) * Q, hot);
 }
 
 // The t-th tile of the launch.  Inside a group: block of m_block token tiles,

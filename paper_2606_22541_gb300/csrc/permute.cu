@@ -492,7 +492,6 @@ cudaError_t launch_dispatch(const void* x, int n, int H, int k, int E, const int
                             int32_t* perm_dst, uint32_t* status, cudaStream_t s) {
   DispatchSeg seg{};
   seg.expert_offsets = offsets;
-  seg.n_chunks_total = ceil_div(n, kChunkTokens);
   seg.rows_total = static_cast<long long>(n) * k;
   return launch_dispatch_seg(x, n, H, k, E, idx, chunk_base, x_perm, perm_src, perm_dst, status, seg, s);
 }
@@ -510,7 +509,6 @@ cudaError_t launch_dispatch_fp8(const void* x, int n, int H, int k, int E, const
                                 cudaStream_t s) {
   DispatchSeg seg{};
   seg.expert_offsets = offsets;
-  seg.n_chunks_total = ceil_div(n, kChunkTokens);
   seg.rows_total = static_cast<long long>(n) * k;
   return launch_dispatch_fp8_seg(x, n, H, k, E, idx, chunk_base, xq, xs, xq_sh, xs_sh, perm_src, perm_dst, status,
                                  seg, s);

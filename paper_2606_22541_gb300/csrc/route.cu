@@ -239,8 +239,7 @@ __global__ void __launch_bounds__(kGateWarps * 32) gate_kernel(const float* logi
                                                                long long plane, int n, GateParams p,
                                                                int32_t* __restrict__ idx,
                                                                float* __restrict__ wout,
-                                                               int32_t* __restrict__ hist, int n_chunks,
-                                                               int chunk0) {
+                                                               int32_t* __restrict__ hist, int chunk0) {
   pdl_wait();
   pdl_launch();
   __shared__ int shist[kMaxExperts];
@@ -831,7 +830,8 @@ cudaError_t launch_router_small(const void* x, const LayerRef& lref, int n, int 
     ASAP_ROUTER_MMA(8)
 #undef ASAP_ROUTER_MMA
   }
-  return launch_pdl(router_small_kernel, ceil_div(n, 8), 256, 0, s, 1, static_cast<const uint4*>(x), lref, status, n, H / 8, E, logits);
+  return launch_pdl(router_small_kernel, ceil_div(n, 8), 256, 0, s, 1, static_cast<const uint4*>(x), lref, status, n,
+                    H / 8, E, logits);
 }
 
 namespace {
@@ -868,21 +868,20 @@ cudaError_t gate_dispatch(const float* logits, int splits, int n, const GatePara
     ASAP_GATE_TEAM(8, 1)
 #undef ASAP_GATE_TEAM
   }
-  return launch_pdl(gate_kernel, ctas, kGateWarps * 32, 0, s, 1, logits, splits, plane, n, p, idx, w, hist, n_chunks,
-                    chunk0);
+  return launch_pdl(gate_kernel, ctas, kGateWarps * 32, 0, s, 1, logits, splits, plane, n, p, idx, w, hist, chunk0);
 }
 }  // namespace
 
 cudaError_t launch_gate(const float* logits, int splits, int n, const GateParams& p, int32_t* idx, float* w,
                         int32_t* hist, cudaStream_t s) {
-  return launch_gate_seg(logits, splits, n, p, idx, w, hist, 0, ceil_div(n, kChunkTokens), s);
+  return launch_gate_seg(logits, splits, n, p, idx, w, hist, 0, s);
 }
 
 cudaError_t launch_gate_seg(const float* logits, int splits, int n, const GateParams& p, int32_t* idx, float* w,
-                            int32_t* hist, int chunk0, int n_chunks_total, cudaStream_t s) {
+                            int32_t* hist, int chunk0, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const int chunks = ceil_div(n, kChunkTokens);
-  return gate_dispatch<false>(logits, splits, n, p, idx, w, hist, chunk0, n_chunks_total, GateScan{}, chunks, s);
+  return gate_dispatch<false>(logits, splits, n, p, idx, w, hist, chunk0, chunks, GateScan{}, chunks, s);
 }
 
 cudaError_t launch_gate_scan(const float* logits, int splits, int n, const GateParams& p, int32_t* idx, float* w,

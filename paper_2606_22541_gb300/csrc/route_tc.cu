@@ -567,7 +567,8 @@ cudaError_t launch_route_fused(const CUtensorMap& tmX, const RouteFusedArgs& a, 
       a.top_k < 1 || a.top_k > kMaxTopK || a.k_iters < a.splits ||
       !(a.seq_slices <= 1 || (a.splits == 1 && (a.seq_slices == 2 || a.seq_slices == 4) && a.k_iters >= a.seq_slices)))
     return cudaErrorInvalidValue;
-  return launch_pdl(route_fused_kernel, dim3(ceil_div(a.n, kGemmBM) * a.splits), dim3(kThreads), kSmem, s, a.splits, tmX, a);
+  return launch_pdl(route_fused_kernel, dim3(ceil_div(a.n, kGemmBM) * a.splits), dim3(kThreads), kSmem, s, a.splits,
+                    tmX, a);
 }
 
 }  // namespace asap
