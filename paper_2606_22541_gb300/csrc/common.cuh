@@ -61,7 +61,7 @@ __device__ __forceinline__ float gate_sigmoid(float l) { return __fdividef(1.0f,
 // waits so, all kernels before that one).  pdl_launch allows the next kernel to
 // start once every CTA has called it or left.  The small kernels call it when
 // their own wait is over, the single-CTA GEMMs when a CTA has no tiles left; the
-// CTA pairs do not (gemm_pair.cu).
+// CTA pairs (gemm_pair.cu) and the CUDA-core router (route.cu) do not.
 //
 // Such a kernel is resident while the data it will read is still being written,
 // so nothing an earlier kernel or the caller writes is read-only for its

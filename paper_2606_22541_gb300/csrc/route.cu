@@ -32,8 +32,7 @@ constexpr int kRouterAhead = 8;  // row pieces in flight per lane
 __global__ void __launch_bounds__(256) router_small_kernel(const uint4* x, LayerRef lref,
                                                            uint32_t* status, int n, int V, int E,
                                                            float* __restrict__ logits) {
-  pdl_wait();
-  pdl_launch();
+  pdl_wait();  // (no pdl_launch: see launch_router_small)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x * 8 + warp;
   if (t >= n) return;
@@ -830,6 +829,10 @@ cudaError_t launch_router_small(const void* x, const LayerRef& lref, int n, int 
     ASAP_ROUTER_MMA(8)
 #undef ASAP_ROUTER_MMA
   }
+  // The gate may not start beside this kernel: its waiting CTAs slowed the last
+  // wave.  asap_moe_route of 4096 tokens, 256 channels: 128 experts 77.8 us with an
+  // early start, 59.5 without (63.5 before dependent launches), 100 experts 68.3 and
+  // 56.3 (60.0); one wave of CTAs (2048 tokens) 47.7 and 45.1.
   return launch_pdl(router_small_kernel, ceil_div(n, 8), 256, 0, s, 1, static_cast<const uint4*>(x), lref, status, n,
                     H / 8, E, logits);
 }
